@@ -143,7 +143,7 @@ __device__ __forceinline__ float2 df_add(float2 x, float2 y) {
   return make_float2(hi, e - (hi - s.x));
 }
 __device__ __forceinline__ float2 df_square(float t) {
-  const float hi = t * t;
+  const float hi = __fmul_rn(t, t);  // not contracted into the sum that follows
   return make_float2(hi, fmaf(t, t, -hi));
 }
 __device__ __forceinline__ float2 warp_sum(float2 v) {

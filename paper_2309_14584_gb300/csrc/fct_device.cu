@@ -389,7 +389,9 @@ size_t team_smem_need(const fct_plan P, int G, bool with_values) {
 
 // Dynamic shared memory of a launch with teams of G blocks that stages only
 // the index tables (batches, serving, the condition probe).
-size_t launch_smem(const fct_plan P, int G, size_t cap) { return std::min(team_smem_need(P, G, false), cap); }
+size_t launch_smem(const fct_plan P, int G, size_t cap) {
+  return std::min(std::max(team_smem_need(P, G, false), static_cast<size_t>(P->hp.tk_smem)), cap);
+}
 
 // Dynamic shared memory a solver block may take without lowering the blocks
 // per SM of the plain kernel (the largest static shared memory of the
@@ -419,6 +421,35 @@ fct_status solver_smem_cap(int bt, const cudaDeviceProp& prop, int* cap_out, int
   return FCT_OK;
 }
 
+// Bytes of the cell tables.
+struct CellBytes {
+  size_t idx = 0, w = 0, dest = 0, wtab = 0, comb = 0, ncomb = 0;
+};
+CellBytes cell_bytes(const CellLayout& L, int K) {
+  const size_t cells = static_cast<size_t>(K) * L.slices, steps = cells * L.blocks * 128;
+  CellBytes b;
+  b.idx = sizeof(uint16_t) * steps;
+  b.w = sizeof(float) * steps;
+  b.dest = sizeof(uint16_t) * cells * L.gmax * 32;
+  b.wtab = sizeof(int2) * cells * (L.warps + 1);
+  b.comb = sizeof(int2) * cells * L.cmax;
+  b.ncomb = sizeof(int32_t) * cells;
+  return b;
+}
+
+// Layout of the mixed path's inner solve by grid groups for a plan with
+// L->rows filled in.
+fct_status choose_cell_layout(fct_plan P, int64_t R, int64_t wave, CellLayout* L) {
+  int dev = 0, cap = 0, per_sm = 0;
+  FCT_CUDA(cudaGetDevice(&dev));
+  cudaDeviceProp prop;
+  FCT_CUDA(cudaGetDeviceProperties(&prop, dev));
+  const fct_status s = solver_smem_cap(P->block_threads, prop, &cap, &per_sm);
+  if (s != FCT_OK) return s;
+  choose_cells(P->N, R, P->K, P->M, P->block_threads, wave, cap, L);
+  return FCT_OK;
+}
+
 fct_status choose_shape(fct_plan P) {
   int dev = 0;
   FCT_CUDA(cudaGetDevice(&dev));
@@ -443,7 +474,9 @@ fct_status choose_shape(fct_plan P) {
   // A single transform on the whole GPU also stages the entry values of the
   // CG loop when every block's share fits (fct_solve_kernel<BT, true>).
   const size_t need_values = team_smem_need(P, P->grid_blocks, true);
-  P->stage_values = need_values <= static_cast<size_t>(cap);
+  // (plans whose inner solve runs by grid groups read the row tables in the
+  // three FP64 sweeps only)
+  P->stage_values = need_values <= static_cast<size_t>(cap) && P->hp.tk_groups == 0;
   P->smem_bytes = static_cast<int>((P->stage_values ? need_values : launch_smem(P, P->grid_blocks, cap)) + 15) & ~15;
   P->smem_bytes = std::min(P->smem_bytes, cap);
   int chk = 0;
@@ -603,6 +636,9 @@ fct_status fct_plan_create(fct_plan* out, int D, int64_t N, const uint16_t* supp
       wave = static_cast<int64_t>(per_sm) * nsm;
   }
   DeviceTables DT;  // device-built tables (scratch, freed on return)
+  CellLayout CL;    // inner solve of the mixed path by grid groups
+  std::vector<char> cell_mem;  // host-built cell tables
+  CellPointers ch{};
   if (on_device) {
     s = build_device_tables(&H, support, sizes, nodes, o.grid_kind, workers, wave, o.entries_per_lane, &epl, &DT,
                             cs);
@@ -614,7 +650,43 @@ fct_status fct_plan_create(fct_plan* out, int D, int64_t N, const uint16_t* supp
     int64_t classes[3][kLaneClasses];
     lane_class_counts(H, classes);
     epl = pick_entries_per_lane(classes, workers, wave, o.entries_per_lane);
+    if (o.precision == FCT_MIXED) {
+      CL.rows.resize(K);
+      for (int l = 0; l < K; ++l) CL.rows[l] = H.row_off[l + 1] - H.row_off[l];
+      s = choose_cell_layout(P, H.R, wave, &CL);
+      if (s != FCT_OK) {
+        delete P;
+        return s;
+      }
+      if (CL.groups > 0) {
+        size_t at = 0;
+        for (int pass = 0; pass < 2; ++pass) {
+          at = 0;
+          auto take = [&](auto** q, size_t bytes) {
+            *q = reinterpret_cast<std::remove_reference_t<decltype(*q)>>(cell_mem.data() + at);
+            at += align256(bytes);
+          };
+          const CellBytes cb = cell_bytes(CL, K);
+          take(&ch.idx, cb.idx);
+          take(&ch.w, cb.w);
+          take(&ch.dest, cb.dest);
+          take(&ch.wtab, cb.wtab);
+          take(&ch.comb, cb.comb);
+          take(&ch.ncomb, cb.ncomb);
+          if (pass == 0) cell_mem.resize(at);
+        }
+        build_cells_host(H, CL, ch);
+      }
+    }
     device_row_order(&H, epl);
+  }
+  if (on_device && o.precision == FCT_MIXED) {
+    CL.rows = DT.grid_rows;
+    s = choose_cell_layout(P, H.R, wave, &CL);
+    if (s != FCT_OK) {
+      delete P;
+      return s;
+    }
   }
   // tensor-core DCT passes: which grids, their A slices and pass lists (may
   // add the identity matrix to the DCT matrices, so before their upload)
@@ -711,6 +783,23 @@ fct_status fct_plan_create(fct_plan* out, int D, int64_t N, const uint16_t* supp
       hp.n_w_units = static_cast<int32_t>((N + hp.w_rows_per_unit - 1) / hp.w_rows_per_unit);
     }
   }
+  if (hp.n_w_units == 0 && CL.groups > 0) {
+    hp.tk_groups = CL.groups;
+    hp.tk_gg = CL.gg;
+    hp.tk_slices = CL.slices;
+    hp.tk_sl = CL.sl;
+    hp.tk_np = CL.np;
+    hp.tk_q = CL.q;
+    hp.tk_ext = CL.ext;
+    hp.tk_blocks = CL.blocks;
+    hp.tk_gmax = CL.gmax;
+    hp.tk_cmax = CL.cmax;
+    hp.tk_cw = CL.cw;
+    hp.tk_lg = CL.lg;
+    hp.tk_nown = CL.nown;
+    hp.tk_smem = CL.smem;
+  }
+  const bool cells = hp.tk_groups > 0;
   const int64_t nnzw = static_cast<int64_t>(w_col.size());
   P->w_rowptr_h = w_rowptr;
 
@@ -752,6 +841,17 @@ fct_status fct_plan_create(fct_plan* out, int D, int64_t N, const uint16_t* supp
   add(&d_wrowptr, sizeof(int32_t) * (nnzw > 0 ? N + 1 : 1));
   add(&d_wcol, sizeof(int32_t) * nnzw);
   add(&d_wval, sizeof(float) * nnzw);
+  const CellBytes cb = cells ? cell_bytes(CL, K) : CellBytes{};
+  CellPointers cp{};
+  int32_t *d_tk_rows, *d_tk_qoff;
+  add(&cp.idx, cb.idx);
+  add(&cp.w, cb.w);
+  add(&cp.dest, cb.dest);
+  add(&cp.wtab, cb.wtab);
+  add(&cp.comb, cb.comb);
+  add(&cp.ncomb, cb.ncomb);
+  add(&d_tk_rows, sizeof(int32_t) * (cells ? K : 0));
+  add(&d_tk_qoff, sizeof(int32_t) * (cells ? K : 0));
   add(&hp.y0, sizeof(double) * std::max<int64_t>(H.M, 1));
   add(&hp.y1, sizeof(double) * std::max<int64_t>(H.M, 1));
   add(&hp.b, sizeof(double) * H.R);
@@ -805,6 +905,14 @@ fct_status fct_plan_create(fct_plan* out, int D, int64_t N, const uint16_t* supp
   hp.crow = d_crow;
   hp.wcm = d_wcm;
   hp.wcm32 = d_wcm32;
+  hp.tk_idx = cp.idx;
+  hp.tk_w = cp.w;
+  hp.tk_dest = cp.dest;
+  hp.tk_wtab = cp.wtab;
+  hp.tk_comb = cp.comb;
+  hp.tk_ncomb = cp.ncomb;
+  hp.tk_rows = d_tk_rows;
+  hp.tk_qoff = d_tk_qoff;
   hp.wrowptr = d_wrowptr;
   hp.wcol = d_wcol;
   hp.wval = d_wval;
@@ -845,6 +953,21 @@ fct_status fct_plan_create(fct_plan* out, int D, int64_t N, const uint16_t* supp
   chk(up(d_crow, on_device ? static_cast<const void*>(DT.crow) : H.crow.data(), sizeof(int32_t) * KN));
   chk(up(d_wcm, on_device ? static_cast<const void*>(DT.wcm) : H.weight.data(), sizeof(double) * KN));
   chk(up(d_wcm32, on_device ? static_cast<const void*>(DT.wcm32) : wc32.data(), sizeof(float) * KN));
+  s = FCT_OK;
+  if (cells) {
+    chk(up(d_tk_rows, CL.rows.data(), sizeof(int32_t) * K));
+    chk(up(d_tk_qoff, CL.qoff.data(), sizeof(int32_t) * K));
+    if (on_device) {
+      s = build_cells_device(DT, N, K, CL, cp);
+    } else {
+      chk(up(cp.idx, ch.idx, cb.idx));
+      chk(up(cp.w, ch.w, cb.w));
+      chk(up(cp.dest, ch.dest, cb.dest));
+      chk(up(cp.wtab, ch.wtab, cb.wtab));
+      chk(up(cp.comb, ch.comb, cb.comb));
+      chk(up(cp.ncomb, ch.ncomb, cb.ncomb));
+    }
+  }
   DT.release();
   if (nnzw > 0) {
     chk(up(d_wrowptr, w_rowptr.data(), sizeof(int32_t) * (N + 1)));
@@ -858,8 +981,7 @@ fct_status fct_plan_create(fct_plan* out, int D, int64_t N, const uint16_t* supp
   chk(up(P->d_support, support, sizeof(uint16_t) * N * D));
   chk(up(P->d_ichunks, H.idct_chunks.data(), sizeof(DctChunk) * H.idct_chunks.size()));
   chk(up(P->d_emats, H.eval_mats.data(), sizeof(double) * H.eval_mats.size()));
-  s = FCT_OK;
-  if (ue == cudaSuccess && P->tc) {
+  if (ue == cudaSuccess && s == FCT_OK && P->tc) {
     std::vector<int32_t> rb, rk;
     final_pass_rows_for(H, P->tc->gfinal, &rb, &rk);
     auto dev = std::make_shared<TcDevice>();

@@ -225,6 +225,30 @@ struct DevPlan {
   const GridFinal* gfinal_tc;
   const int32_t* rowbase_tc;
   const int32_t* rowk_tc;
+  // inner solve by grid groups (fct_cells.cuh); tk_groups = 0: not used
+  int32_t tk_groups;         // tasks: groups of tk_gg consecutive grids
+  int32_t tk_gg;
+  int32_t tk_slices;         // slices of tk_sl coefficients; cell l * tk_slices + s is one (grid, slice)
+  int32_t tk_sl;
+  int64_t tk_np;             // = tk_slices * tk_sl: stride of the tasks' t vectors
+  int32_t tk_q;              // floats of a group's row sums in shared memory
+  int32_t tk_ext;            // extra slots of a grid, after its rows (runs of rows cut into several)
+  int32_t tk_blocks;         // allocated blocks of four steps, groups and cut rows per cell
+  int32_t tk_gmax;
+  int32_t tk_cmax;
+  int32_t tk_cw;             // owner chunks: coefficients per chunk, threads per coefficient, chunks
+  int32_t tk_lg;
+  int32_t tk_nown;
+  int32_t tk_smem;           // shared memory the inner solve needs (bytes)
+  int32_t pad_tk;
+  const uint16_t* tk_idx;    // [cells][tk_blocks][32][4] coefficient inside the slice; bit 15: a group ends
+  const float* tk_w;         // [cells][tk_blocks][32][4] entry values
+  const uint16_t* tk_dest;   // [cells][tk_gmax][32] where a run's sum goes: row, or extra slot
+  const int2* tk_wtab;       // [cells][warps + 1] first block and first group of each warp
+  const int2* tk_comb;       // [cells][tk_cmax] rows of several runs: row | runs << 16, first extra slot
+  const int32_t* tk_ncomb;   // [cells]
+  const int32_t* tk_rows;    // [K] rows of the grid
+  const int32_t* tk_qoff;    // [K] start of the grid's row sums inside its group's
 };
 
 // One transform of a launch.
@@ -349,6 +373,11 @@ struct DeviceTables {
   int32_t* crow = nullptr;     // [K N] coefficient-major
   double* wcm = nullptr;
   float* wcm32 = nullptr;
+  int32_t* col0 = nullptr;     // [K N] columns, rows in bin order (before the solver row order)
+  int32_t* crow0 = nullptr;    // [K N] coefficient-major rows, bin order
+  int32_t* scratch[4] = {nullptr, nullptr, nullptr, nullptr};  // [K N] each, free once the tables are built
+  int32_t* grows = nullptr;        // [K] rows of each grid
+  std::vector<int32_t> grid_rows;  // the same on the host
   void* stream = nullptr;      // cudaStream_t of the build: allocation and release are ordered on it
   void release();
   ~DeviceTables() { release(); }
@@ -389,6 +418,33 @@ void device_row_order(HostTables* H, int epl);
 // A p gather units for `workers` threads per block: a unit holds
 // workers / lanes consecutive rows of equal lane count.
 void row_units(const HostTables& H, int workers, int epl, std::vector<int32_t>* first, std::vector<int32_t>* lanes);
+
+// Layout of the inner solve by grid groups (fct_cells.cuh).
+struct CellLayout {
+  int32_t groups = 0, gg = 0, slices = 0, sl = 0, warps = 0;
+  int64_t np = 0;
+  int32_t q = 0, ext = 0, blocks = 0, gmax = 0, cmax = 0, cw = 0, lg = 0, nown = 0, smem = 0;
+  std::vector<int32_t> rows, qoff;  // [K]
+};
+constexpr int kCellRun = 32;          // longest run of a row
+constexpr int kCellMaxSlice = 32736;  // 15-bit coefficient index, 32 padding slots included
+// Chooses the layout from the rows of every grid (L->rows), the block size,
+// the co-resident blocks `wave`, the shared memory `cap` a block may take and
+// the M doubles of each DCT buffer.  groups stays 0 where it does not fit.
+void choose_cells(int64_t N, int64_t R, int K, int64_t M, int block_threads, int64_t wave, int cap, CellLayout* L);
+// Cell tables (see DevPlan).  The device build takes the build's pre-order
+// tables and is ordered on its stream; the host build takes H before
+// device_row_order and fills host arrays of the same sizes.  Both give the
+// same arrays.
+struct CellPointers {
+  uint16_t* idx;
+  float* w;
+  uint16_t* dest;
+  int2 *wtab, *comb;
+  int32_t* ncomb;
+};
+fct_status build_cells_device(const DeviceTables& T, int64_t N, int K, const CellLayout& L, const CellPointers& out);
+void build_cells_host(const HostTables& H, const CellLayout& L, const CellPointers& out);
 
 // W = A^T A (N x N, CSR, columns ascending, FP64 sums in a fixed order) and
 // the bound sum over rows of A of (row length)^2 >= nnz(W), cheap to compute

@@ -429,6 +429,223 @@ __global__ void final_rows_kernel(int64_t R, const int32_t* __restrict__ rowsrc,
   }
 }
 
+// Rows of every grid: its CSR entries are l N .. l N + N - 1 (one per column),
+// rows ascending.
+__global__ void grid_rows_kernel(int K, int64_t N, const int32_t* __restrict__ col0,
+                                 const int32_t* __restrict__ crow0, int32_t* __restrict__ rows) {
+  const int l = blockIdx.x * blockDim.x + threadIdx.x;
+  if (l >= K) return;
+  const int64_t b = l * N;
+  rows[l] = crow0[b + col0[b + N - 1]] - crow0[b + col0[b]] + 1;
+}
+
+// Cell tables (DevPlan): one cell (grid l, slice s) per block.
+//   1. the grid's columns in row order that fall in the slice (a stable
+//      selection), as (row, coefficient) pairs in `ent`;
+//   2. their rows: start of each in `start`, rows counted by a scan of the marks
+//      of a row's first entry; run lengths into a histogram;
+//   3. groups of 32 runs, longest first: steps before each group (`goff`), the
+//      warps' shares, padding everywhere;
+//   4. each row's place: rank of its first full run (`rfull`) and of its last run
+//      (`rlast`) in the order by length, rows ascending within a length;
+//   5. every entry to its run's lane and step; run destinations; end marks.
+// The block works tile after tile, so no other block is involved; ent, start,
+// rfull, rlast and goff are the cell's share of build scratch ([K N] each).
+constexpr int kCellWarpsMax = 16;
+struct CellArgs {
+  int64_t N;
+  int S, SL, NW, blocks, gmax, cmax, ext;
+  const int32_t* col0;
+  const int32_t* crow0;
+  const float* wcm32;
+  const int32_t* rows;
+  int32_t *ent, *start, *rfull, *rlast;
+  int32_t* goff;  // [cells][gmax + 1]
+  CellPointers out;
+};
+__global__ void __launch_bounds__(kScanThreads) cell_build_kernel(const CellArgs a) {
+  __shared__ int32_t hist[kCellRun + 1], base[kCellRun + 1], seen[kCellRun + 1];
+  __shared__ int32_t wcnt[kScanThreads / 32][kCellRun + 1];
+  __shared__ int32_t gb[kCellWarpsMax + 1], sb[kCellWarpsMax + 1];
+  const int64_t cell = blockIdx.x, l = cell / a.S;
+  const int s = static_cast<int>(cell % a.S);
+  const int64_t m0 = static_cast<int64_t>(s) * a.SL;
+  const int n = static_cast<int>(min(static_cast<int64_t>(a.SL), a.N - m0));
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int32_t* col = a.col0 + l * a.N;
+  const int32_t* crow = a.crow0 + l * a.N;
+  const int32_t r0 = crow[col[0]], nrow = a.rows[l];
+  uint32_t* ent = reinterpret_cast<uint32_t*>(a.ent) + l * a.N + m0;
+  int32_t* start = a.start + l * a.N + m0;
+  int32_t* rfull = a.rfull + l * a.N + m0;
+  int32_t* rlast = a.rlast + l * a.N + m0;
+  int32_t* goff = a.goff + cell * (a.gmax + 1);
+  int32_t total;
+  // 1. selection
+  int32_t run = 0;
+  for (int64_t j0 = 0; j0 < a.N; j0 += kScanTile) {
+    int32_t c[kScanItems];
+    int32_t cnt = 0;
+#pragma unroll
+    for (int k = 0; k < kScanItems; ++k) {
+      const int64_t j = j0 + static_cast<int64_t>(t) * kScanItems + k;
+      c[k] = j < a.N ? col[j] : -1;
+      const int64_t v = c[k] - m0;
+      if (v < 0 || v >= n) c[k] = -1;
+      cnt += c[k] >= 0;
+    }
+    int32_t pos = run + block_exclusive_scan(cnt, &total);
+#pragma unroll
+    for (int k = 0; k < kScanItems; ++k)
+      if (c[k] >= 0)
+        ent[pos++] = (static_cast<uint32_t>(crow[c[k]] - r0) << 16) | static_cast<uint32_t>(c[k] - m0);
+    run += total;
+  }
+  if (t <= kCellRun) hist[t] = seen[t] = 0;
+  __syncthreads();
+  // 2. rows
+  int32_t nslot = 0;
+  for (int j0 = 0; j0 < n; j0 += kScanThreads) {
+    const int j = j0 + t;
+    const bool head = j < n && (j == 0 || (ent[j] >> 16) != (ent[j - 1] >> 16));
+    const int32_t pos = nslot + block_exclusive_scan(head ? 1 : 0, &total);
+    if (head) start[pos] = j;
+    nslot += total;
+  }
+  __syncthreads();
+  auto row_len = [&](int i) { return (i + 1 < nslot ? start[i + 1] : n) - start[i]; };
+  int32_t nfull = 0;  // full runs that are not their row's last
+  for (int i0 = 0; i0 < nslot; i0 += kScanThreads) {
+    const int i = i0 + t;
+    int32_t nf = 0;
+    if (i < nslot) {
+      const int32_t len = row_len(i);
+      nf = (len - 1) / kCellRun;
+      atomicAdd(&hist[len - nf * kCellRun], 1);
+    }
+    const int32_t pos = nfull + block_exclusive_scan(nf, &total);
+    if (i < nslot) rfull[i] = pos;
+    nfull += total;
+  }
+  __syncthreads();
+  // 3. groups
+  if (t == 0) {
+    int32_t b = 0;
+    for (int k = kCellRun; k >= 1; --k) {
+      base[k] = b;
+      b += hist[k] + (k == kCellRun ? nfull : 0);
+    }
+    base[0] = b;
+    seen[kCellRun] = nfull;  // the last runs of full length follow the others
+  }
+  __syncthreads();
+  const int nrun = base[0], G = (nrun + 31) / 32;
+  int32_t steps = 0;
+  for (int g0 = 0; g0 < G; g0 += kScanThreads) {
+    const int g = g0 + t;
+    int32_t len = 0;
+    if (g < G) {
+      len = kCellRun;
+      while (len > 1 && 32 * g >= base[len - 1]) --len;
+    }
+    const int32_t pos = steps + block_exclusive_scan(len, &total);
+    if (g < G) goff[g] = pos;
+    steps += total;
+  }
+  if (t == 0) goff[G] = steps;
+  if (t <= kCellWarpsMax) gb[t] = G;
+  __syncthreads();
+  auto warp_of = [&](int g) {
+    return static_cast<int>(min(static_cast<int64_t>(a.NW - 1), static_cast<int64_t>(goff[g]) * a.NW / steps));
+  };
+  for (int g = t; g < G; g += kScanThreads) {
+    const int w = warp_of(g);
+    for (int k = g == 0 ? 0 : warp_of(g - 1) + 1; k <= w; ++k) gb[k] = g;
+  }
+  __syncthreads();
+  if (t == 0) {
+    sb[0] = 0;
+    for (int w = 0; w < a.NW; ++w) sb[w + 1] = sb[w] + (goff[gb[w + 1]] - goff[gb[w]] + 3) / 4;
+  }
+  __syncthreads();
+  if (t <= a.NW) a.out.wtab[cell * (a.NW + 1) + t] = make_int2(sb[t], gb[t]);
+  uint16_t* idx = a.out.idx + cell * a.blocks * 128;
+  float* wv = a.out.w + cell * a.blocks * 128;
+  uint16_t* dest = a.out.dest + cell * a.gmax * 32;
+  for (int i = t; i < sb[a.NW] * 128; i += kScanThreads) {
+    idx[i] = static_cast<uint16_t>(a.SL + ((i >> 2) & 31));
+    wv[i] = 0.0f;
+  }
+  for (int i = t; i < min(G + 2, a.gmax) * 32; i += kScanThreads) dest[i] = static_cast<uint16_t>(nrow + a.ext);
+  // 4. places of the rows' last runs; cut rows
+  int32_t next = 0, ncomb = 0;
+  for (int i0 = 0; i0 < nslot; i0 += kScanThreads) {
+    const int i = i0 + t;
+    int32_t len = 0, nf = 0, tail = 0;
+    if (i < nslot) {
+      len = row_len(i);
+      nf = (len - 1) / kCellRun;
+      tail = len - nf * kCellRun;
+    }
+    const unsigned peers = __match_any_sync(0xffffffffu, tail);
+    for (int k = t; k < (kScanThreads / 32) * (kCellRun + 1); k += kScanThreads) wcnt[k / (kCellRun + 1)][k % (kCellRun + 1)] = 0;
+    __syncthreads();
+    if (tail > 0 && (peers & ((1u << lane) - 1u)) == 0) wcnt[warp][tail] = __popc(peers);
+    __syncthreads();
+    if (t >= 1 && t <= kCellRun) {
+      int32_t r = seen[t];
+      for (int w = 0; w < kScanThreads / 32; ++w) {
+        const int32_t c = wcnt[w][t];
+        wcnt[w][t] = r;
+        r += c;
+      }
+      seen[t] = r;
+    }
+    __syncthreads();
+    if (i < nslot) rlast[i] = base[tail] + wcnt[warp][tail] + __popc(peers & ((1u << lane) - 1u));
+    const int32_t e = next + block_exclusive_scan(nf > 0 ? nf + 1 : 0, &total);
+    next += total;
+    const int32_t ci = ncomb + block_exclusive_scan(nf > 0 ? 1 : 0, &total);
+    ncomb += total;
+    if (i < nslot) {
+      const int32_t row = static_cast<int32_t>(ent[start[i]] >> 16);
+      if (nf > 0) {
+        a.out.comb[cell * a.cmax + ci] = make_int2(row | ((nf + 1) << 16), nrow + e);
+        for (int k = 0; k < nf; ++k) dest[rfull[i] + k] = static_cast<uint16_t>(nrow + e + k);
+      }
+      dest[rlast[i]] = static_cast<uint16_t>(nf > 0 ? nrow + e + nf : row);
+    }
+  }
+  if (t == 0) a.out.ncomb[cell] = ncomb;
+  __syncthreads();
+  // 5. entries
+  auto place = [&](int32_t rank, int k) {
+    const int g = rank >> 5;
+    const int w = warp_of(g);
+    const int st = goff[g] - goff[gb[w]] + k;
+    return (static_cast<int64_t>(sb[w] + (st >> 2)) * 32 + (rank & 31)) * 4 + (st & 3);
+  };
+  int32_t before = 0;
+  for (int j0 = 0; j0 < n; j0 += kScanThreads) {
+    const int j = j0 + t;
+    const bool head = j < n && (j == 0 || (ent[j] >> 16) != (ent[j - 1] >> 16));
+    const int32_t i = before + block_exclusive_scan(head ? 1 : 0, &total) + (head ? 1 : 0) - 1;
+    before += total;
+    if (j < n) {
+      const int32_t pos = j - start[i], nf = (row_len(i) - 1) / kCellRun, ch = pos / kCellRun;
+      const int64_t at = place(ch < nf ? rfull[i] + ch : rlast[i], pos - ch * kCellRun);
+      const int32_t c = static_cast<int32_t>(ent[j] & 0xffffu);
+      idx[at] = static_cast<uint16_t>(c);
+      wv[at] = a.wcm32[l * a.N + m0 + c];
+    }
+  }
+  __syncthreads();
+  for (int i = t; i < G * 32; i += kScanThreads) {
+    const int64_t at = place(i, goff[(i >> 5) + 1] - goff[i >> 5] - 1);
+    idx[at] |= 0x8000u;
+  }
+}
+
 __global__ void set_int_kernel(int32_t* dst, int32_t v) { *dst = v; }
 
 fct_status cuda_err(cudaError_t e, const char* what) {
@@ -501,7 +718,7 @@ fct_status build_device_tables(HostTables* Hp, const uint16_t* support, const in
   auto add = [&](void* dst, size_t bytes) { pieces.push_back({reinterpret_cast<void**>(dst), bytes}); };
   uint16_t* d_support;
   int32_t *d_sizes, *d_strides, *d_k0, *d_v0, *d_k1, *d_v1, *d_ghist, *d_part, *d_small;
-  int32_t *d_rowptr0, *d_rowsrc0, *d_rowgrid0, *d_col0, *d_crow0, *d_inv, *d_rowsrc, *d_nzoff;
+  int32_t *d_rowptr0, *d_rowsrc0, *d_rowgrid0, *d_col0, *d_crow0, *d_inv, *d_rowsrc, *d_nzoff, *d_grows;
   uint32_t* d_pairs;
   double *d_nodes, *d_weight, *d_wcsr0;
   int64_t* d_offsets;
@@ -526,6 +743,7 @@ fct_status build_device_tables(HostTables* Hp, const uint16_t* support, const in
   add(&d_rowsrc0, sizeof(int32_t) * KN);
   add(&d_rowgrid0, sizeof(int32_t) * KN);
   add(&d_col0, sizeof(int32_t) * KN);
+  add(&d_grows, sizeof(int32_t) * K);
   add(&d_wcsr0, sizeof(double) * KN);
   add(&d_crow0, sizeof(int32_t) * KN);
   add(&d_inv, sizeof(int32_t) * KN);
@@ -555,6 +773,13 @@ fct_status build_device_tables(HostTables* Hp, const uint16_t* support, const in
     }
   }
   out->wcm = d_weight;  // the coefficient-major values are the fold's output
+  out->col0 = d_col0;
+  out->crow0 = d_crow0;
+  out->grows = d_grows;
+  out->scratch[0] = d_k0;
+  out->scratch[1] = d_v0;
+  out->scratch[2] = d_k1;
+  out->scratch[3] = d_v1;
 
   cudaError_t ue = cudaSuccess;
   auto chk = [&](cudaError_t x) {
@@ -607,6 +832,9 @@ fct_status build_device_tables(HostTables* Hp, const uint16_t* support, const in
     return fail(FCT_ERR_CUDA, "device table build: row count out of range");
   }
 
+  grid_rows_kernel<<<elem_blocks(K), kElemThreads, 0, st>>>(K, N, d_col0, d_crow0, d_grows);
+  out->grid_rows.assign(K, 0);
+  chk(cudaMemcpyAsync(out->grid_rows.data(), d_grows, sizeof(int32_t) * K, cudaMemcpyDeviceToHost, st));
   // entries per lane from the lane-class histogram
   chk(cudaMemsetAsync(d_small, 0, sizeof(int32_t) * 32, st));
   lane_class_kernel<<<elem_blocks(R), kElemThreads, 0, st>>>(d_rowptr0, R, d_small);
@@ -657,6 +885,37 @@ fct_status build_device_tables(HostTables* Hp, const uint16_t* support, const in
     return fail(FCT_ERR_CUDA, "device table build: inconsistent row pointer");
   }
   return FCT_OK;
+}
+
+fct_status build_cells_device(const DeviceTables& T, int64_t N, int K, const CellLayout& L, const CellPointers& o) {
+  const cudaStream_t st = static_cast<cudaStream_t>(T.stream);
+  CellArgs a;
+  a.N = N;
+  a.S = L.slices;
+  a.SL = L.sl;
+  a.NW = L.warps;
+  a.blocks = L.blocks;
+  a.gmax = L.gmax;
+  a.cmax = L.cmax;
+  a.ext = L.ext;
+  a.col0 = T.col0;
+  a.crow0 = T.crow0;
+  a.wcm32 = T.wcm32;
+  a.rows = T.grows;
+  a.ent = T.scratch[0];
+  a.start = T.scratch[1];
+  a.rfull = T.scratch[2];
+  a.rlast = T.scratch[3];
+  a.out = o;
+  const int64_t cells = static_cast<int64_t>(K) * L.slices;
+  void* goff = nullptr;
+  cudaError_t e = cudaMallocAsync(&goff, sizeof(int32_t) * cells * (L.gmax + 1), st);
+  if (e != cudaSuccess) return cuda_err(e, "cudaMallocAsync(cell tables)");
+  a.goff = static_cast<int32_t*>(goff);
+  cell_build_kernel<<<static_cast<unsigned>(cells), kScanThreads, 0, st>>>(a);
+  e = cudaGetLastError();
+  cudaFreeAsync(goff, st);
+  return e == cudaSuccess ? FCT_OK : cuda_err(e, "cell tables");
 }
 
 fct_status download_device_tables(const DeviceTables& T, HostTables* Hp) {

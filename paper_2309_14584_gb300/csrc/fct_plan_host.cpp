@@ -544,6 +544,152 @@ void normal_matrix(const HostTables& H, std::vector<int32_t>* rowptr, std::vecto
   }
 }
 
+void choose_cells(int64_t N, int64_t R, int K, int64_t M, int block_threads, int64_t wave, int cap, CellLayout* L) {
+  L->groups = 0;
+  if (wave < 1) wave = 1;
+  if (R < N) return;  // rank-deficient; the solver keeps an N-vector in the row workspace
+  L->qoff.assign(K, 0);
+  L->warps = block_threads / 32;
+  const int64_t ncap = (N + 31) / 32 * 32;
+  // one task per co-resident block: as many grids per group as that takes;
+  // fewer where a group's row sums leave no room for a slice
+  for (int gg = static_cast<int>((K + wave - 1) / wave); gg >= 1; gg = gg > 1 ? gg / 2 : 0) {
+    // the slice and the extra slots (2 per kCellRun coefficients and grid)
+    // share the room the rows leave
+    int64_t rmax = 0;
+    for (int l0 = 0; l0 < K; l0 += gg) {
+      int64_t q = 0;
+      for (int l = l0; l < std::min(K, l0 + gg); ++l) q += (3 * L->rows[l]) / 2 + 72;
+      rmax = std::max(rmax, q);
+    }
+    const int64_t room = cap / 4 - rmax - 64;
+    int64_t sl = room * 64 / (64 + 6 * gg);
+    sl = std::min({sl, ncap, static_cast<int64_t>(kCellMaxSlice)}) / 32 * 32;
+    if (sl < std::min<int64_t>(ncap, 2048)) continue;
+    const int64_t S = (N + sl - 1) / sl;
+    sl = ((N + S - 1) / S + 31) / 32 * 32;
+    if ((S - 1) * sl >= N) continue;
+    const int64_t NG = (K + gg - 1) / gg, np = S * sl;
+    const int64_t ext = 2 * (sl / kCellRun) + 2;
+    int64_t qmax = 0;
+    bool fits = true;
+    for (int l0 = 0; l0 < K; l0 += gg) {
+      int64_t q = 0;
+      for (int l = l0; l < std::min(K, l0 + gg); ++l) {
+        L->qoff[l] = static_cast<int32_t>(q);
+        // row sums, then the run destinations (16 bits; up to 31 idle lanes in
+        // the last group and two groups after it)
+        q += (L->rows[l] + ext + 1 + 3) / 4 * 4 + ((L->rows[l] + ext + 31) / 32 + 2) * 16;
+        fits = fits && L->rows[l] + ext + 1 <= 65535;
+      }
+      qmax = std::max(qmax, q);
+    }
+    const int64_t smem = 4 * (qmax + sl + 32);
+    // owner chunks: as many coefficients as spread N over the wave, the block's
+    // other threads taking shares of the groups
+    int64_t cw = ((N + wave - 1) / wave + 31) / 32 * 32;
+    cw = std::min<int64_t>(cw, block_threads);
+    const int64_t nown = (N + cw - 1) / cw;
+    if (!fits || smem > cap || NG * np * 4 > M * 8 || (NG + 2 * nown) * 8 > M * 8) continue;
+    L->gg = gg;
+    L->groups = static_cast<int32_t>(NG);
+    L->slices = static_cast<int32_t>(S);
+    L->sl = static_cast<int32_t>(sl);
+    L->np = np;
+    L->q = static_cast<int32_t>(qmax);
+    L->ext = static_cast<int32_t>(ext);
+    // sorted by length, 32 to a group, padding is at most kCellRun steps; each
+    // warp's share is padded to four
+    L->blocks = static_cast<int32_t>((sl / 32 + kCellRun + 1 + 3 * L->warps + 3) / 4 + 1);
+    L->gmax = static_cast<int32_t>(sl / 32 + 3);
+    L->cmax = static_cast<int32_t>(sl / kCellRun + 1);
+    L->cw = static_cast<int32_t>(cw);
+    L->lg = static_cast<int32_t>(block_threads / cw);
+    L->nown = static_cast<int32_t>(nown);
+    L->smem = std::max<int32_t>(static_cast<int32_t>(smem), 4 * block_threads);  // the owner chunks' sums
+    return;
+  }
+}
+
+void build_cells_host(const HostTables& H, const CellLayout& L, const CellPointers& o) {
+  const int64_t N = H.N, SL = L.sl;
+  const int S = L.slices, NW = L.warps;
+  struct Run {
+    int32_t start, len, dest;
+  };
+  std::vector<std::vector<int32_t>> cols(S);
+  for (int64_t l = 0; l < H.K; ++l) {
+    const int32_t r0 = H.row_off[l], nrow = L.rows[l];
+    for (auto& c : cols) c.clear();
+    for (int64_t j = 0; j < N; ++j) cols[H.col[l * N + j] / SL].push_back(H.col[l * N + j]);
+    for (int s = 0; s < S; ++s) {
+      const int64_t cell = l * S + s;
+      const std::vector<int32_t>& c = cols[s];
+      const int n = static_cast<int>(c.size());
+      auto row_of = [&](int j) { return H.crow[l * N + c[j]] - r0; };
+      // runs by length: the full runs of long rows first, then every row's last
+      std::vector<std::vector<Run>> full(kCellRun + 1), last(kCellRun + 1);
+      int32_t ext = 0, ncomb = 0;
+      for (int j = 0; j < n;) {
+        int e = j;
+        while (e < n && row_of(e) == row_of(j)) ++e;
+        const int len = e - j, nf = (len - 1) / kCellRun;
+        for (int k = 0; k < nf; ++k) full[kCellRun].push_back({j + k * kCellRun, kCellRun, nrow + ext + k});
+        const int tail = len - nf * kCellRun;
+        last[tail].push_back({j + nf * kCellRun, tail, nf > 0 ? nrow + ext + nf : row_of(j)});
+        if (nf > 0) {
+          o.comb[cell * L.cmax + ncomb++] = int2{row_of(j) | ((nf + 1) << 16), nrow + ext};
+          ext += nf + 1;
+        }
+        j = e;
+      }
+      o.ncomb[cell] = ncomb;
+      std::vector<Run> runs;
+      for (int k = kCellRun; k >= 1; --k) {
+        runs.insert(runs.end(), full[k].begin(), full[k].end());
+        runs.insert(runs.end(), last[k].begin(), last[k].end());
+      }
+      const int G = static_cast<int>((runs.size() + 31) / 32);
+      std::vector<int32_t> off(G + 1, 0);
+      for (int g = 0; g < G; ++g) off[g + 1] = off[g] + runs[32 * g].len;
+      std::vector<int32_t> gb(NW + 1, G), sb(NW + 1, 0);
+      for (int g = G - 1; g >= 0; --g) {
+        const int w = static_cast<int>(std::min<int64_t>(NW - 1, static_cast<int64_t>(off[g]) * NW / off[G]));
+        for (int k = g == 0 ? 0 : static_cast<int>(std::min<int64_t>(NW - 1, static_cast<int64_t>(off[g - 1]) * NW / off[G])) + 1;
+             k <= w; ++k)
+          gb[k] = g;
+      }
+      for (int w = 0; w < NW; ++w) sb[w + 1] = sb[w] + (off[gb[w + 1]] - off[gb[w]] + 3) / 4;
+      for (int w = 0; w <= NW; ++w) o.wtab[cell * (NW + 1) + w] = int2{sb[w], gb[w]};
+      uint16_t* idx = o.idx + cell * L.blocks * 128;
+      float* wv = o.w + cell * L.blocks * 128;
+      uint16_t* dest = o.dest + cell * L.gmax * 32;
+      for (int b = 0; b < sb[NW]; ++b)
+        for (int i = 0; i < 128; ++i) {
+          idx[b * 128 + i] = static_cast<uint16_t>(SL + i / 4);
+          wv[b * 128 + i] = 0.0f;
+        }
+      for (int i = 0; i < std::min(G + 2, L.gmax) * 32; ++i) dest[i] = static_cast<uint16_t>(nrow + L.ext);
+      for (int w = 0; w < NW; ++w)
+        for (int g = gb[w]; g < gb[w + 1]; ++g)
+          for (int k = 0; k < off[g + 1] - off[g]; ++k) {
+            const int st = off[g] - off[gb[w]] + k;
+            for (int i = 0; i < 32; ++i) {
+              const int64_t at = ((sb[w] + st / 4) * 32 + i) * 4 + st % 4;
+              const int r = 32 * g + i;
+              if (r < static_cast<int>(runs.size()) && k < runs[r].len) {
+                const int32_t m = c[runs[r].start + k];
+                idx[at] = static_cast<uint16_t>(m - s * SL);
+                wv[at] = static_cast<float>(H.weight[l * N + m]);
+              }
+              if (k + 1 == off[g + 1] - off[g]) idx[at] |= 0x8000u;
+            }
+          }
+      for (int r = 0; r < static_cast<int>(runs.size()); ++r) dest[r] = static_cast<uint16_t>(runs[r].dest);
+    }
+  }
+}
+
 void final_pass_rows_for(const HostTables& H, const std::vector<GridFinal>& gfinal, std::vector<int32_t>* rowbase,
                          std::vector<int32_t>* rowk) {
   rowbase->resize(H.R);

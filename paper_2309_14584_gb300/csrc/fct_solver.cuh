@@ -41,7 +41,7 @@ __device__ __forceinline__ int wt_start(int off, int n) { return (off + n + 1) &
 //   8-byte aligned after the indices.
 template <int BT>
 __device__ void load_block_tabs(const DevPlan& P, const Team& tm, unsigned char* dsm, int smem_bytes, BlockTabs* T,
-                                bool with_w, int wbytes) {
+                                bool with_w, int wbytes, bool stage) {
   const int nru = P.n_row_units, ncc = P.n_coef_chunks, nwu = with_w ? P.n_w_units : 0;
   const int nA = nru > tm.rank ? (nru - tm.rank + tm.G - 1) / tm.G : 0;
   const int nB = ncc > tm.rank ? (ncc - tm.rank + tm.G - 1) / tm.G : 0;
@@ -62,7 +62,7 @@ __device__ void load_block_tabs(const DevPlan& P, const Team& tm, unsigned char*
   int* hdrW = hdrB + nB;
   const int nhdr = (5 * nA + nB + 2 * nW + 1) & ~1;  // the pool starts 8-byte aligned
   int* pool = hdrA + nhdr;
-  const int cap = (smem_bytes - off) / 4 - nhdr;  // ints left for the pool
+  const int cap = stage ? (smem_bytes - off) / 4 - nhdr : 0;  // ints left for the pool
   const int wi = wbytes / 4;  // ints per staged entry value
   int used = 0, cachedA = 0, cachedB = 0, cachedW = 0;
   if (cap > 0) {
@@ -618,6 +618,7 @@ __device__ __forceinline__ bool coef_owner(const DevPlan& P, int c, int wk, int*
 // ---------------------------------------------------------------------------
 constexpr int kUnitGroup = 16;  // units per flush of the per-warp partials
 
+#include "fct_cells.cuh"
 
 template <int BT, typename V, typename WT, typename XT, bool SV, int DEEP>
 __device__ bool cg_normal(const DevPlan& P, Team& tm, const BlockTabs& T, const WT* wcsr, const WT* wcm,
@@ -1079,9 +1080,16 @@ __device__ bool solve_job(const SolveJob& J, Team& tm, double* red, unsigned cha
     if (threadIdx.x == 0) atomicExch(tm.err, static_cast<int>(FCT_ERR_INVALID_ARG));
     return false;
   }
+  // the inner solve by grid groups takes the whole of the block's shared memory
+  // once b is known, so nothing but the DCT matrices is staged for it
+  const bool cells = !SV && J.precision == FCT_MIXED && P.tk_groups > 0 && P.s_init == nullptr;
+  if (cells && smem_bytes < P.tk_smem) {  // the host sizes launches to hold it
+    if (threadIdx.x == 0) atomicExch(tm.err, static_cast<int>(FCT_ERR_INVALID_ARG));
+    return false;
+  }
   BlockTabs T;
   load_block_tabs<BT>(P, tm, dsm, smem_bytes, &T, J.precision == FCT_MIXED && P.n_w_units > 0 && P.s_init == nullptr,
-                      SV ? (J.precision == FCT_MIXED ? 4 : 8) : 0);
+                      SV ? (J.precision == FCT_MIXED ? 4 : 8) : 0, !cells);
   const int ncc = P.n_coef_chunks, nre = P.n_rowel_chunks, nru = P.n_row_units, nwide = P.n_wide_units;
   const int wk = static_cast<int>(threadIdx.x) - 32;
   const int nce = (P.N + BT - 1) / BT;  // elementwise units over coefficients
@@ -1160,7 +1168,9 @@ __device__ bool solve_job(const SolveJob& J, Team& tm, double* red, unsigned cha
     for (int u = tm.rank; u < nce; u += tm.G) {
       const int m = u * BT + threadIdx.x;
       if (m < P.N) {
-        stcg(P.sp32 + m, make_float2(static_cast<float>(ldcg(P.sp + m).x * ci), 0.0f));
+        const float v = static_cast<float>(ldcg(P.sp + m).x * ci);
+        if (cells) stcg(reinterpret_cast<float*>(P.sp32) + m, v);  // cg_cells keeps s contiguous
+        else stcg(P.sp32 + m, make_float2(v, 0.0f));
         stcg(P.dx32 + m, 0.0f);
       }
     }
@@ -1173,6 +1183,11 @@ __device__ bool solve_job(const SolveJob& J, Team& tm, double* red, unsigned cha
       if (P.n_w_units > 0) {
         if (!pcg_normal_w<BT>(P, tm, T, g64 * ci * ci, J.inner_tol, J.max_iter, 64, &it_in, &g_in, &st_in))
           return false;
+      } else if (cells) {
+        if constexpr (!SV) {
+          if (!cg_cells<BT>(P, tm, dsm, g64 * ci * ci, J.inner_tol, J.max_iter, 64, &it_in, &g_in, &st_in))
+            return false;
+        }
       } else if (!cg_normal<BT, float, float, float, SV, DEEP>(P, tm, T, P.wcsr32, P.wcm32, P.sp32, P.q32, P.dx32,
                                                      g64 * ci * ci, J.inner_tol, J.max_iter, 64, &it_in, &g_in,
                                                      &st_in, red)) {
@@ -1211,7 +1226,8 @@ __device__ bool solve_job(const SolveJob& J, Team& tm, double* red, unsigned cha
         t = coef_combine<BT / 32 - 1>(P, T, t, kc, wk, m, &lead);
         double part = 0.0;
         if (lead) {
-          stcg(P.sp32 + m, make_float2(static_cast<float>(t * ci), 0.0f));
+          if (cells) stcg(reinterpret_cast<float*>(P.sp32) + m, static_cast<float>(t * ci));
+          else stcg(P.sp32 + m, make_float2(static_cast<float>(t * ci), 0.0f));
           stcg(P.sp + m, make_double2(t, 0.0));  // for an FP64 continuation
           stcg(P.dx32 + m, 0.0f);
           part = t * t;
