@@ -7,23 +7,22 @@
 // that holds s (or a slice of it) and q_l in shared memory does both, and only
 // the sum over grids t = sum_l t_l and the vector updates cross blocks.
 //
-// The iteration is the form of CG with one point of reduction (Chronopoulos
-// and Gear): the operator is applied to the residual s, not to p, so phase 1
-// needs no scalar and reads 4 bytes per coefficient:
-//   phase 1, per task (a group of tk_gg grids, one block): q_l = A_l s and
-//     delta = |q|^2, then t = sum_{l in group} A_l^T q_l, streamed out (tpart);
-//   phase 2, per owner chunk: gamma = |s|^2, beta = gamma / gamma_prev,
-//     alpha = gamma / (delta - beta gamma / alpha_prev);
-//     p = s + beta p, z = t + beta z, x += alpha p, s -= alpha z.
-// Two team barriers per iteration, as in cg_normal, but every scattered access
-// is to shared memory and global traffic is coalesced: 6 bytes of table per
-// entry (read by the gather and again, from L2, by the scatter).
+// Per iteration (s = residual of the normal equations, as in cg_normal):
+//   phase 1, per task (a group of tk_gg grids, one block): p = s + beta p_old
+//     into shared memory, q_l = A_l p and |q|^2, then t = sum_{l in group}
+//     A_l^T q_l, streamed out (tpart);
+//   phase 2, per owner chunk: t = sum over groups of tpart, then x += alpha p,
+//     s -= alpha t.
+// Two team barriers, as in cg_normal, but every scattered access is to shared
+// memory and global traffic is coalesced: 6 bytes of table per entry (read by
+// the gather and again, from L2, by the scatter) and 8 + 4 bytes of vectors per
+// coefficient and task.
 //
 // Cell tables.  A cell is one (grid, slice of tk_sl coefficients).  Its rows are
 // cut into runs of at most kCellRun entries, sorted by length, 32 to a group:
 // lane i of a warp sums run i of the group, one entry a step, so a step is 32
 // independent entries and pads are few (sorted lengths).  A warp's groups are
-// contiguous, so it streams its steps, four at a time, without looking at group
+// contiguous, so it streams its steps, four to a block, without looking at group
 // boundaries ahead: bit 15 of a step's indices marks the last step of a group,
 // where the lanes store their sums and go on to the next 32 runs.  Rows of
 // several runs are completed by cell_join.  The order of additions depends only
@@ -33,24 +32,24 @@
 
 #include "fct_common.cuh"
 
-__device__ __forceinline__ float2 df_mul(float2 a, float2 b) {
-  const float p = __fmul_rn(a.x, b.x);
-  const float e = fmaf(a.x, b.x, -p) + fmaf(a.x, b.y, __fmul_rn(a.y, b.x));
-  const float hi = p + e;
-  return make_float2(hi, e - (hi - p));
+__device__ __forceinline__ uint32_t shared_addr(const void* p) {
+  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
-__device__ __forceinline__ float2 df_div(float2 a, float2 b) {
-  const float q1 = __fdividef(a.x, b.x);
-  const float2 qb = df_mul(make_float2(q1, 0.0f), b);
-  const float2 r = df_add(a, make_float2(-qb.x, -qb.y));
-  const float q2 = __fdividef(r.x, b.x);
-  const float hi = q1 + q2;
-  return make_float2(hi, q2 - (hi - q1));
+__device__ __forceinline__ float lds_f32(uint32_t a) {
+  float v;
+  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a));
+  return v;
 }
-
+__device__ __forceinline__ uint32_t lds_u16(uint32_t a) {
+  uint16_t v;
+  asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ void sts_f32(uint32_t a, float v) {
+  asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+}
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
-  const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(shared_addr(dst)), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
@@ -58,225 +57,328 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_al
 // for idle lanes), then the run destinations of the cell at hand.
 __device__ __forceinline__ int cell_q_floats(int rows, int ext) { return (rows + ext + 1 + 3) & ~3; }
 
-struct CellView {  // one cell, as its warp sees it
-  const uint2* idx;       // [blocks][32] four steps per lane
-  const float4* w;
-  const uint16_t* dest;   // shared, [groups][32], this lane's
-  int b0, b1;             // this warp's blocks of four steps
-};
-
-template <int NW>
-__device__ __forceinline__ CellView cell_view(const DevPlan& P, int cell, const uint16_t* dest) {
-  const int warp = static_cast<int>(threadIdx.x >> 5), lane = threadIdx.x & 31;
-  CellView v;
-  const int2* wt = P.tk_wtab + static_cast<int64_t>(cell) * (NW + 1) + warp;
-  const int2 a = __ldg(wt), b = __ldg(wt + 1);
-  v.b0 = a.x;
-  v.b1 = b.x;
-  const int64_t base = static_cast<int64_t>(cell) * P.tk_blocks * 32 + lane;
-  v.idx = reinterpret_cast<const uint2*>(P.tk_idx) + base;
-  v.w = reinterpret_cast<const float4*>(P.tk_w) + base;
-  v.dest = dest + a.y * 32 + lane;
-  return v;
-}
-
-// Run destinations of a cell into shared memory (asynchronous copies; two
-// groups of idle destinations follow the last).
+// Run destinations of a cell into shared memory (asynchronous copies; kCellIdle
+// groups of idle destinations follow the last: they are read ahead).
 template <int NW>
 __device__ __forceinline__ void cell_load_dest(const DevPlan& P, int cell, uint16_t* dest) {
-  const int n16 = (__ldg(P.tk_wtab + static_cast<int64_t>(cell) * (NW + 1) + NW).y + 2) * 4;
+  const int n16 = (__ldg(P.tk_wtab + static_cast<int64_t>(cell) * (NW + 1) + NW).y + kCellIdle) * 4;
   const uint16_t* src = P.tk_dest + static_cast<int64_t>(cell) * P.tk_gmax * 32;
   for (int i = threadIdx.x; i < n16; i += NW * 32) cp_async16(dest + 8 * i, src + 8 * i);
 }
 
+// A step's index is the coefficient in the slice (15 bits) and the mark; the
+// byte offset in shared memory is 4 x the coefficient.
+__device__ __forceinline__ uint32_t cell_at0(uint32_t v) { return (v & 0x7fffu) << 2; }
+__device__ __forceinline__ uint32_t cell_at1(uint32_t v) { return (v >> 14) & 0x1fffcu; }
+
 constexpr int kCellAhead = 4;  // blocks of four steps a warp keeps in flight
 
-// q[dest] (+)= the sums of w s over the cell's runs.  ADD: the plan has several
-// slices, whose sums add up in q.
-template <int NW, bool ADD>
-__device__ __forceinline__ void cell_gather(const CellView& v, const float* s, float* q) {
-  if (v.b0 >= v.b1) return;
+// Calls block(indices, values) for the n blocks of four steps of a warp's share of
+// a cell, kCellAhead loaded ahead.
+template <typename Block>
+__device__ __forceinline__ void cell_stream(const uint2* __restrict__ idx, const float4* __restrict__ w, int n,
+                                            Block block) {
   uint2 in[kCellAhead];
   float4 wn[kCellAhead];
 #pragma unroll
   for (int j = 0; j < kCellAhead; ++j) {
-    const int b = min(v.b0 + j, v.b1 - 1);
-    in[j] = __ldg(v.idx + b * 32);
-    wn[j] = __ldg(v.w + b * 32);
+    const int b = min(j, n - 1);
+    in[j] = __ldg(idx + b * 32);
+    wn[j] = __ldg(w + b * 32);
   }
-  const uint16_t* dp = v.dest;
-  float acc = 0.0f;
-  for (int b = v.b0; b < v.b1; b += kCellAhead) {
+  int b = 0;
+#pragma unroll 1
+  for (; b + kCellAhead <= n; b += kCellAhead) {
+    uint2 ic[kCellAhead];
+    float4 wc[kCellAhead];
 #pragma unroll
     for (int j = 0; j < kCellAhead; ++j) {
-      if (b + j >= v.b1) continue;
-      const uint2 ic = in[j];
-      const float4 wc = wn[j];
-      const int nb = min(b + kCellAhead + j, v.b1 - 1);
-      in[j] = __ldg(v.idx + nb * 32);
-      wn[j] = __ldg(v.w + nb * 32);
-      const float s0 = s[ic.x & 0x7fffu], s1 = s[(ic.x >> 16) & 0x7fffu];
-      const float s2 = s[ic.y & 0x7fffu], s3 = s[(ic.y >> 16) & 0x7fffu];
-      auto end = [&](uint32_t mark) {
-        if (mark) {  // the same for all lanes
-          const int d = *dp;
-          if (ADD) q[d] += acc;
-          else q[d] = acc;
-          acc = 0.0f;
-          dp += 32;
-        }
-      };
-      acc = fmaf(wc.x, s0, acc);
-      if (((ic.x | ic.y) & 0x80008000u) == 0) {  // no run ends here
-        acc = fmaf(wc.y, s1, acc);
-        acc = fmaf(wc.z, s2, acc);
-        acc = fmaf(wc.w, s3, acc);
-      } else {
-        end(ic.x & 0x8000u);
-        acc = fmaf(wc.y, s1, acc);
-        end(ic.x & 0x80000000u);
-        acc = fmaf(wc.z, s2, acc);
-        end(ic.y & 0x8000u);
-        acc = fmaf(wc.w, s3, acc);
-        end(ic.y & 0x80000000u);
-      }
+      ic[j] = in[j];
+      wc[j] = wn[j];
     }
+#pragma unroll
+    for (int j = 0; j < kCellAhead; ++j) {
+      const int nb = min(b + kCellAhead + j, n - 1);
+      in[j] = __ldg(idx + nb * 32);
+      wn[j] = __ldg(w + nb * 32);
+    }
+#pragma unroll
+    for (int j = 0; j < kCellAhead; ++j) block(ic[j], wc[j]);
   }
+#pragma unroll
+  for (int j = 0; j < kCellAhead - 1; ++j)
+    if (b + j < n) block(in[j], wn[j]);
 }
 
-// t[m] (+)= w q[row] over the cell's entries.  Every column has one entry per
+// q[dest] (+)= the sums of w p over n blocks of a cell.  ADD: the plan has
+// several slices, whose sums add up in q.  sp, sq, sd: shared addresses of the
+// slice of p, the grid's row sums and this lane's first destination.  A run's
+// place (and, with ADD, its sum so far) is loaded while the runs before it are
+// summed: the chain of loads per ending run would bound cells of short rows.
+// Its own function (not inlined): the loop needs its registers for the loads in
+// flight.
+template <bool ADD>
+__device__ __noinline__ void cell_gather(const uint2* __restrict__ idx, const float4* __restrict__ w, int n,
+                                         uint32_t sp, uint32_t sq, uint32_t sd) {
+  float acc = 0.0f;
+  uint32_t a = sq + 4 * lds_u16(sd), an = sq + 4 * lds_u16(sd + 64);
+  float old = ADD ? lds_f32(a) : 0.0f;
+  sd += 128;
+  auto end = [&](uint32_t mark) {
+    if (mark) {  // the same for all lanes
+      sts_f32(a, ADD ? old + acc : acc);
+      acc = 0.0f;
+      a = an;
+      if (ADD) old = lds_f32(a);
+      an = sq + 4 * lds_u16(sd);
+      sd += 64;
+    }
+  };
+  cell_stream(idx, w, n, [&](uint2 ic, float4 wc) {
+    const float p0 = lds_f32(sp + cell_at0(ic.x)), p1 = lds_f32(sp + cell_at1(ic.x));
+    const float p2 = lds_f32(sp + cell_at0(ic.y)), p3 = lds_f32(sp + cell_at1(ic.y));
+    acc = fmaf(wc.x, p0, acc);
+    if (((ic.x | ic.y) & 0x80008000u) == 0) {  // no run ends here
+      acc = fmaf(wc.y, p1, acc);
+      acc = fmaf(wc.z, p2, acc);
+      acc = fmaf(wc.w, p3, acc);
+    } else {
+      end(ic.x & 0x8000u);
+      acc = fmaf(wc.y, p1, acc);
+      end(ic.x & 0x80000000u);
+      acc = fmaf(wc.z, p2, acc);
+      end(ic.y & 0x8000u);
+      acc = fmaf(wc.w, p3, acc);
+      end(ic.y & 0x80000000u);
+    }
+  });
+}
+
+// t[m] (+)= w q[row] over n blocks of a cell.  Every column has one entry per
 // grid, so no two entries of a cell touch the same t; the first grid of a group
 // stores, the others add.
-template <int NW, bool ADD>
-__device__ __forceinline__ void cell_scatter(const CellView& v, const float* q, float* t) {
-  if (v.b0 >= v.b1) return;
-  uint2 in[kCellAhead];
-  float4 wn[kCellAhead];
-#pragma unroll
-  for (int j = 0; j < kCellAhead; ++j) {
-    const int b = min(v.b0 + j, v.b1 - 1);
-    in[j] = __ldg(v.idx + b * 32);
-    wn[j] = __ldg(v.w + b * 32);
-  }
-  const uint16_t* dp = v.dest;
-  float qv = q[*dp];
-  for (int b = v.b0; b < v.b1; b += kCellAhead) {
-#pragma unroll
-    for (int j = 0; j < kCellAhead; ++j) {
-      if (b + j >= v.b1) continue;
-      const uint2 ic = in[j];
-      const float4 wc = wn[j];
-      const int nb = min(b + kCellAhead + j, v.b1 - 1);
-      in[j] = __ldg(v.idx + nb * 32);
-      wn[j] = __ldg(v.w + nb * 32);
-      const uint32_t a0 = ic.x & 0x7fffu, a1 = (ic.x >> 16) & 0x7fffu, a2 = ic.y & 0x7fffu, a3 = (ic.y >> 16) & 0x7fffu;
-      float t0 = 0.0f, t1 = 0.0f, t2 = 0.0f, t3 = 0.0f;
-      if (ADD) {  // the four entries of a lane are different columns
-        t0 = t[a0];
-        t1 = t[a1];
-        t2 = t[a2];
-        t3 = t[a3];
-      }
-      auto next = [&](uint32_t mark) {
-        if (mark) {
-          dp += 32;
-          qv = q[*dp];
-        }
-      };
-      auto term = [&](float w, float old) { return ADD ? fmaf(w, qv, old) : w * qv; };
-      t0 = term(wc.x, t0);
-      if (((ic.x | ic.y) & 0x80008000u) == 0) {
-        t1 = term(wc.y, t1);
-        t2 = term(wc.z, t2);
-        t3 = term(wc.w, t3);
-      } else {
-        next(ic.x & 0x8000u);
-        t1 = term(wc.y, t1);
-        next(ic.x & 0x80000000u);
-        t2 = term(wc.z, t2);
-        next(ic.y & 0x8000u);
-        t3 = term(wc.w, t3);
-        next(ic.y & 0x80000000u);
-      }
-      t[a0] = t0;
-      t[a1] = t1;
-      t[a2] = t2;
-      t[a3] = t3;
+template <bool ADD>
+__device__ __noinline__ void cell_scatter(const uint2* __restrict__ idx, const float4* __restrict__ w, int n,
+                                          uint32_t sv, uint32_t sq, uint32_t sd) {
+  float qv = lds_f32(sq + 4 * lds_u16(sd)), qn = lds_f32(sq + 4 * lds_u16(sd + 64));
+  uint32_t an = sq + 4 * lds_u16(sd + 128);
+  sd += 192;
+  auto next = [&](uint32_t mark) {
+    if (mark) {
+      qv = qn;
+      qn = lds_f32(an);
+      an = sq + 4 * lds_u16(sd);
+      sd += 64;
     }
-  }
+  };
+  cell_stream(idx, w, n, [&](uint2 ic, float4 wc) {
+    const uint32_t a0 = sv + cell_at0(ic.x), a1 = sv + cell_at1(ic.x), a2 = sv + cell_at0(ic.y), a3 = sv + cell_at1(ic.y);
+    float t0 = 0.0f, t1 = 0.0f, t2 = 0.0f, t3 = 0.0f;
+    if (ADD) {  // the four entries of a lane are different columns
+      t0 = lds_f32(a0);
+      t1 = lds_f32(a1);
+      t2 = lds_f32(a2);
+      t3 = lds_f32(a3);
+    }
+    auto term = [&](float wv, float before) { return ADD ? fmaf(wv, qv, before) : __fmul_rn(wv, qv); };
+    t0 = term(wc.x, t0);
+    if (((ic.x | ic.y) & 0x80008000u) == 0) {
+      t1 = term(wc.y, t1);
+      t2 = term(wc.z, t2);
+      t3 = term(wc.w, t3);
+    } else {
+      next(ic.x & 0x8000u);
+      t1 = term(wc.y, t1);
+      next(ic.x & 0x80000000u);
+      t2 = term(wc.z, t2);
+      next(ic.y & 0x8000u);
+      t3 = term(wc.w, t3);
+      next(ic.y & 0x80000000u);
+    }
+    sts_f32(a0, t0);
+    sts_f32(a1, t1);
+    sts_f32(a2, t2);
+    sts_f32(a3, t3);
+  });
 }
 
-// Rows of several runs: their runs' sums sit in q at extra slots; a warp adds
-// them in a fixed order.  One slice (ADD = false): the total is the row's sum,
-// written back to the extra slots for the scatter.  Several: it is added to the
-// row, and cell_spread writes the finished row back before the scatter.
+// Rows of several runs: their runs' sums sit in q at extra slots; a thread adds
+// up to kCellFew of them, a warp more, in a fixed order.  One slice (ADD =
+// false): the total is the row's sum, written back to the extra slots for the
+// scatter.  Several: it is added to the row, the extra slots are cleared for the
+// next slice, and cell_spread writes the finished row back before the scatter.
+// Few-run rows fill tk_comb from its end, the others from its start.
 template <int NW, bool ADD>
 __device__ __forceinline__ void cell_join(const DevPlan& P, int cell, float* q) {
   const int warp = static_cast<int>(threadIdx.x >> 5), lane = threadIdx.x & 31;
-  const int n = __ldg(P.tk_ncomb + cell);
+  const int2 n = __ldg(P.tk_ncomb + cell);
   const int2* cb = P.tk_comb + static_cast<int64_t>(cell) * P.tk_cmax;
-  for (int i = warp; i < n; i += NW) {
+  for (int i = threadIdx.x; i < n.y; i += NW * 32) {
+    const int2 c = __ldg(cb + P.tk_cmax - 1 - i);
+    const int row = c.x & 0xffff, cnt = (c.x >> 16) & 0xffff;
+    float v = 0.0f;
+    for (int e = 0; e < cnt; ++e) v += q[c.y + e];
+    for (int e = 0; e < cnt; ++e) q[c.y + e] = ADD ? 0.0f : v;
+    if (ADD) q[row] += v;
+    else q[row] = v;
+  }
+  for (int i = warp; i < n.x; i += NW) {
     const int2 c = __ldg(cb + i);
     const int row = c.x & 0xffff, cnt = (c.x >> 16) & 0xffff;
     float v = 0.0f;
     for (int e = lane; e < cnt; e += 32) v += q[c.y + e];
     v = warp_sum(v);
-    if (ADD) {
-      if (lane == 0) q[row] += v;
-    } else {
-      for (int e = lane; e < cnt; e += 32) q[c.y + e] = v;
-      if (lane == 0) q[row] = v;
+    for (int e = lane; e < cnt; e += 32) q[c.y + e] = ADD ? 0.0f : v;
+    if (lane == 0) {
+      if (ADD) q[row] += v;
+      else q[row] = v;
     }
   }
 }
 template <int NW>
 __device__ __forceinline__ void cell_spread(const DevPlan& P, int cell, float* q) {
   const int warp = static_cast<int>(threadIdx.x >> 5), lane = threadIdx.x & 31;
-  const int n = __ldg(P.tk_ncomb + cell);
+  const int2 n = __ldg(P.tk_ncomb + cell);
   const int2* cb = P.tk_comb + static_cast<int64_t>(cell) * P.tk_cmax;
-  for (int i = warp; i < n; i += NW) {
+  for (int i = threadIdx.x; i < n.y; i += NW * 32) {
+    const int2 c = __ldg(cb + P.tk_cmax - 1 - i);
+    const float v = q[c.x & 0xffff];
+    for (int e = 0; e < ((c.x >> 16) & 0xffff); ++e) q[c.y + e] = v;
+  }
+  for (int i = warp; i < n.x; i += NW) {
     const int2 c = __ldg(cb + i);
     const float v = q[c.x & 0xffff];
     for (int e = lane; e < ((c.x >> 16) & 0xffff); e += 32) q[c.y + e] = v;
   }
 }
 
-// Warp 0: the double-float sums of two lists of partials (every lane).
-__device__ __forceinline__ void warp0_sum2(const float2* a, int na, const float2* b, int nb, float2* sa, float2* sb) {
-  float2 va = make_float2(0.0f, 0.0f), vb = va;
-  for (int i0 = threadIdx.x; i0 < max(na, nb); i0 += 32 * 8) {
-    float2 ta[8], tb[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int i = i0 + 32 * j;
-      ta[j] = i < na ? ldcg(a + i) : make_float2(0.0f, 0.0f);
-      tb[j] = i < nb ? ldcg(b + i) : make_float2(0.0f, 0.0f);
+// Phase 1 of one task: the grids l0 .. l0 + ng - 1.  p = s + beta p_old (s at the
+// first iteration) slice by slice, the grids' row sums, |q|^2 (scaled by rsf;
+// this thread's compensated share is returned), and t of every coefficient to
+// tp.  Its own function (not inlined) for its registers; all threads call it, and
+// it ends with a block barrier.
+template <int BT>
+__device__ __noinline__ float2 cells_task(const DevPlan& P, unsigned char* dsm, int l0, int ng, float beta, bool first,
+                                          float rsf, float* tp) {
+  constexpr int NW = BT / 32;
+  const int tid = static_cast<int>(threadIdx.x), warp = tid >> 5, lane = tid & 31;
+  const int N = P.N, S = P.tk_slices, SL = P.tk_sl, l1 = l0 + ng;
+  float* const qs = reinterpret_cast<float*>(dsm);  // [tk_q] row sums and destinations of the grids
+  float* const vs = qs + P.tk_q;                    // [SL + 32] the slice of p, then of t
+  const float* const sv = reinterpret_cast<const float*>(P.sp32);
+  const float* const pv = sv + ((N + 3) & ~3);
+  auto q_of = [&](int l) { return qs + __ldg(P.tk_qoff + l); };
+  auto dest_of = [&](int l) {
+    return reinterpret_cast<uint16_t*>(q_of(l) + cell_q_floats(__ldg(P.tk_rows + l), P.tk_ext));
+  };
+  // a cell's row sums, this lane's first destination and this warp's blocks;
+  // loaded one cell ahead
+  struct Geom {
+    const uint2* idx;
+    const float4* w;
+    int n;
+    uint32_t sq, sd;
+  };
+  auto geom = [&](int l, int s) {
+    const int2* wt = P.tk_wtab + static_cast<int64_t>(l * S + s) * (NW + 1) + warp;
+    const int2 a = __ldg(wt);
+    const int off = __ldg(P.tk_qoff + l), rows = __ldg(P.tk_rows + l);
+    Geom g;
+    const int64_t at = (static_cast<int64_t>(l * S + s) * P.tk_blocks + a.x) * 32 + lane;
+    g.idx = reinterpret_cast<const uint2*>(P.tk_idx) + at;
+    g.w = reinterpret_cast<const float4*>(P.tk_w) + at;
+    g.n = __ldg(&wt[1].x) - a.x;
+    g.sq = shared_addr(qs + off);
+    g.sd = g.sq + 4 * cell_q_floats(rows, P.tk_ext) + (a.y * 32 + lane) * 2;
+    return g;
+  };
+  const uint32_t sp = shared_addr(vs);
+  if (S > 1) {
+    for (int i = tid; i < P.tk_q; i += BT) qs[i] = 0.0f;
+    __syncthreads();  // the copies below write the destinations in between
+  }
+  for (int l = l0; l < l1; ++l) cell_load_dest<NW>(P, l * S, dest_of(l));
+  for (int s = 0; s < S; ++s) {
+    const int m0 = s * SL, n = min(SL, N - m0);
+    if (s > 0) {
+      for (int l = l0; l < l1; ++l) cell_load_dest<NW>(P, l * S + s, dest_of(l));
     }
-#pragma unroll
-    for (int o = 4; o > 0; o >>= 1)
-#pragma unroll
-      for (int j = 0; j < o; ++j) {
-        ta[j] = df_add(ta[j], ta[j + o]);
-        tb[j] = df_add(tb[j], tb[j + o]);
+    Geom cur = geom(l0, s);
+    if (first) {
+#pragma unroll 4
+      for (int i = 4 * tid; i < n; i += 4 * BT)
+        *reinterpret_cast<float4*>(vs + i) = ldcg(reinterpret_cast<const float4*>(sv + m0 + i));
+    } else {
+#pragma unroll 4
+      for (int i = 4 * tid; i < n; i += 4 * BT) {
+        const float4 a = ldcg(reinterpret_cast<const float4*>(sv + m0 + i));
+        const float4 b = ldcg(reinterpret_cast<const float4*>(pv + m0 + i));
+        *reinterpret_cast<float4*>(vs + i) =
+            make_float4(fmaf(beta, b.x, a.x), fmaf(beta, b.y, a.y), fmaf(beta, b.z, a.z), fmaf(beta, b.w, a.w));
       }
-    va = df_add(va, ta[0]);
-    vb = df_add(vb, tb[0]);
+    }
+    if (tid < 32) vs[SL + tid] = 0.0f;  // what padding entries read
+    cp_async_wait();
+    __syncthreads();
+    for (int l = l0; l < l1; ++l) {
+      const Geom g = cur;
+      if (l + 1 < l1) cur = geom(l + 1, s);
+      if (g.n == 0) continue;
+      if (S > 1) cell_gather<true>(g.idx, g.w, g.n, sp, g.sq, g.sd);
+      else cell_gather<false>(g.idx, g.w, g.n, sp, g.sq, g.sd);
+    }
+    __syncthreads();
+    for (int l = l0; l < l1; ++l) {
+      if (S > 1) cell_join<NW, true>(P, l * S + s, q_of(l));
+      else cell_join<NW, false>(P, l * S + s, q_of(l));
+    }
+    __syncthreads();
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    va = df_add(va, make_float2(__shfl_xor_sync(0xffffffffu, va.x, o), __shfl_xor_sync(0xffffffffu, va.y, o)));
-    vb = df_add(vb, make_float2(__shfl_xor_sync(0xffffffffu, vb.x, o), __shfl_xor_sync(0xffffffffu, vb.y, o)));
+  // |q|^2: compensated sums of exact squares
+  float hi = 0.0f, lo = 0.0f;
+  for (int l = l0; l < l1; ++l) {
+    const float* q = q_of(l);
+    const int nr = __ldg(P.tk_rows + l);
+    for (int i = tid; i < nr; i += BT) {
+      const float2 sq = df_square(q[i] * rsf);
+      const float2 t = df_two_sum(hi, sq.x);
+      hi = t.x;
+      lo += t.y + sq.y;
+    }
   }
-  *sa = va;
-  *sb = vb;
+  // t = sum over the grids of A_l^T q_l
+  for (int s = 0; s < S; ++s) {
+    const int m0 = s * SL, n = min(SL, N - m0);
+    Geom cur = geom(l0, s);
+    if (S > 1) {
+      for (int l = l0; l < l1; ++l) cell_load_dest<NW>(P, l * S + s, dest_of(l));
+      for (int l = l0; l < l1; ++l) cell_spread<NW>(P, l * S + s, q_of(l));
+      cp_async_wait();
+      __syncthreads();
+    }
+    for (int l = l0; l < l1; ++l) {
+      const Geom g = cur;
+      if (l + 1 < l1) cur = geom(l + 1, s);
+      if (g.n > 0) {
+        if (l == l0) cell_scatter<false>(g.idx, g.w, g.n, sp, g.sq, g.sd);
+        else cell_scatter<true>(g.idx, g.w, g.n, sp, g.sq, g.sd);
+      }
+      __syncthreads();
+    }
+    for (int i = 4 * tid; i < n; i += 4 * BT)
+      stcg(reinterpret_cast<float4*>(tp + m0 + i), *reinterpret_cast<const float4*>(vs + i));
+    __syncthreads();
+  }
+  return df_two_sum(hi, lo);
 }
 
 // CG on A^T A d = g by grid groups (see the head of this file).  On entry
 // s = right-hand side, x = 0, gamma0 = |s|^2; returns as cg_normal does.  s and p
-// are the halves of sp32, z is q32, tpart lives in y0 and the per-task and
-// per-chunk partials in y1 (the DCT's buffers, free by now).
+// are the halves of sp32, tpart lives in y0 and the per-task and per-chunk
+// partials in y1 (the DCT's buffers, free by now).
+// Not inlined: the calls inside would cost the solver's other paths registers.
 template <int BT>
-__device__ bool cg_cells(const DevPlan& P, Team& tm, unsigned char* dsm, double gamma0, double tol, int max_iter,
+__device__ __noinline__ bool cg_cells(const DevPlan& P, Team& team, unsigned char* dsm, double gamma0, double tol, int max_iter,
                          int stall, int* iters_out, double* gamma_out, int* status_out) {
   constexpr int NW = BT / 32;
   __shared__ float2 wpart[kUnitGroup][NW];
@@ -290,18 +392,16 @@ __device__ bool cg_cells(const DevPlan& P, Team& tm, unsigned char* dsm, double 
     if (!isfinite(gamma0)) *status_out = FCT_ERR_NONFINITE;
     return true;
   }
-  const int N = P.N, K = P.K, NG = P.tk_groups, GG = P.tk_gg, S = P.tk_slices, SL = P.tk_sl;
+  const int N = P.N, K = P.K, NG = P.tk_groups, GG = P.tk_gg;
+  Team tm = team;  // its fields in registers
   const int64_t NP = P.tk_np;
   const int CW = P.tk_cw, LG = P.tk_lg, nown = P.tk_nown;
-  const int tid = static_cast<int>(threadIdx.x), warp = tid >> 5;
-  float* const qs = reinterpret_cast<float*>(dsm);  // [tk_q] row sums of the group's grids
-  float* const vs = qs + P.tk_q;                    // [SL + 32] the slice of s, then of t
+  const int tid = static_cast<int>(threadIdx.x), warp = tid >> 5, lane = tid & 31;
   float* const tpart = reinterpret_cast<float*>(P.y0);
   float2* const part_r = reinterpret_cast<float2*>(P.y1);
   float2* const part_c = part_r + NG;
   float* const sv = reinterpret_cast<float*>(P.sp32);
-  float* const pv = sv + N;
-  float* const zv = P.q32;
+  float* const pv = sv + ((N + 3) & ~3);
   float* const xv = P.dx32;
   int e0 = 0;
   frexp(gamma0, &e0);
@@ -310,98 +410,59 @@ __device__ bool cg_cells(const DevPlan& P, Team& tm, unsigned char* dsm, double 
   const double c0 = gamma0 * rs * rs;
   const float tol2 = static_cast<float>(tol * tol * c0);
   // thread 0's state, in scaled units
-  const float2 g0 = make_float2(static_cast<float>(c0), static_cast<float>(c0 - static_cast<float>(c0)));
-  float2 gam_prev = g0, al_prev = make_float2(1.0f, 0.0f), gam = g0;
-  float best = 3.0e38f;
-  int best_it = 0;
-  auto dest_of = [&](int l) {
-    return reinterpret_cast<uint16_t*>(qs + __ldg(P.tk_qoff + l) + cell_q_floats(__ldg(P.tk_rows + l), P.tk_ext));
-  };
+  float2 gam = df_of(c0);
+  float best = gam.x;
+  int best_it = 0, it = 0;
+  bool first = true;
   auto flush = [&](float2* part, int u0, int nk) {
     __syncthreads();
     if (tid < nk) {
-      float2 v = make_float2(0.0f, 0.0f);
-#pragma unroll
-      for (int w = 0; w < NW; ++w) v = padd(v, wpart[tid][w]);
-      stcg(part + u0 + tid * tm.G, v);
+      stcg(part + u0 + tid * tm.G, warps_sum<NW>(wpart[tid]));
     }
     __syncthreads();
   };
-  int ctl = 0, it = 0;
-  for (;; ++it) {
+  int ctl = 0;
+  for (;;) {
     // ================= phase 1
     {
-      int kg = 0, u0 = tm.rank;
-      for (int g = tm.rank; g < NG; g += tm.G) {
-        const int l0 = g * GG, l1 = min(K, l0 + GG);
-        if (S > 1) {
-          for (int i = tid; i < P.tk_q; i += BT) qs[i] = 0.0f;
-          __syncthreads();  // the copies below write the destinations in between
-        }
-        for (int s = 0; s < S; ++s) {
-          const int m0 = s * SL, n = min(SL, N - m0);
-          for (int i = 4 * tid; i < n; i += 4 * BT) cp_async16(vs + i, sv + m0 + i);
-          for (int l = l0; l < l1; ++l) cell_load_dest<NW>(P, l * S + s, dest_of(l));
-          if (tid < 32) vs[SL + tid] = 0.0f;  // what padding entries read
-          cp_async_wait();
-          __syncthreads();
-          for (int l = l0; l < l1; ++l) {
-            const CellView v = cell_view<NW>(P, l * S + s, dest_of(l));
-            float* q = qs + __ldg(P.tk_qoff + l);
-            if (S > 1) cell_gather<NW, true>(v, vs, q);
-            else cell_gather<NW, false>(v, vs, q);
-          }
-          __syncthreads();
-          for (int l = l0; l < l1; ++l) {
-            float* q = qs + __ldg(P.tk_qoff + l);
-            if (S > 1) cell_join<NW, true>(P, l * S + s, q);
-            else cell_join<NW, false>(P, l * S + s, q);
-          }
-          if (S > 1) {  // the next slice uses the extra slots again
-            __syncthreads();
-            for (int l = l0; l < l1; ++l) {
-              float* q = qs + __ldg(P.tk_qoff + l) + __ldg(P.tk_rows + l);
-              for (int i = tid; i < P.tk_ext; i += BT) q[i] = 0.0f;
+      if (warp == 0) {
+        float2 gnew = gam;
+        if (!first) gnew = warp0_sum(part_c, nown);
+        if (tid == 0) {
+          int c = 0;
+          float bt = 0.0f;
+          if (!first) {
+            ++it;
+            if (!isfinite(gnew.x)) {
+              c = FCT_ERR_NONFINITE + 16;
+            } else {
+              bt = df_div(gnew, gam).x;
+              gam = gnew;
+              if (gam.x <= tol2) c = 1;
+              else if (it >= max_iter) c = FCT_ERR_NOCONV + 16;
+              else if (stall > 0) {
+                if (gam.x < best) {
+                  best = gam.x;
+                  best_it = it;
+                } else if (it - best_it >= stall) {
+                  c = 1;
+                }
+              }
             }
           }
+          sh_ab[1] = bt;
+          sh_ctl[0] = c;
         }
-        __syncthreads();
-        // delta: compensated sums of exact squares
-        float hi = 0.0f, lo = 0.0f;
-        for (int l = l0; l < l1; ++l) {
-          const float* q = qs + __ldg(P.tk_qoff + l);
-          const int nr = __ldg(P.tk_rows + l);
-          for (int i = tid; i < nr; i += BT) {
-            const float2 sq = df_square(q[i] * rsf);
-            const float2 t = df_two_sum(hi, sq.x);
-            hi = t.x;
-            lo += t.y + sq.y;
-          }
-        }
-        const float2 part = warp_sum(df_two_sum(hi, lo));
-        if ((tid & 31) == 0) wpart[kg][warp] = part;
-        // t = sum over the group's grids of A_l^T q_l
-        float* tp = tpart + g * NP;
-        for (int s = 0; s < S; ++s) {
-          const int m0 = s * SL, n = min(SL, N - m0);
-          if (S > 1) {
-            for (int l = l0; l < l1; ++l) cell_load_dest<NW>(P, l * S + s, dest_of(l));
-            for (int l = l0; l < l1; ++l) cell_spread<NW>(P, l * S + s, qs + __ldg(P.tk_qoff + l));
-            if (tid < 32) vs[SL + tid] = 0.0f;
-            cp_async_wait();
-            __syncthreads();
-          }
-          for (int l = l0; l < l1; ++l) {
-            const CellView v = cell_view<NW>(P, l * S + s, dest_of(l));
-            const float* q = qs + __ldg(P.tk_qoff + l);
-            if (l == l0) cell_scatter<NW, false>(v, q, vs);
-            else cell_scatter<NW, true>(v, q, vs);
-            __syncthreads();
-          }
-          for (int i = 4 * tid; i < n; i += 4 * BT)
-            stcg(reinterpret_cast<float4*>(tp + m0 + i), *reinterpret_cast<const float4*>(vs + i));
-          __syncthreads();
-        }
+      }
+      __syncthreads();
+      ctl = sh_ctl[0];
+      if (ctl != 0) break;
+      const float beta = sh_ab[1];
+      int kg = 0, u0 = tm.rank;
+      for (int g = tm.rank; g < NG; g += tm.G) {
+        const int l0 = g * GG;
+        const float2 part = warp_sum(cells_task<BT>(P, dsm, l0, min(K, l0 + GG) - l0, beta, first, rsf, tpart + g * NP));
+        if (lane == 0) wpart[kg][warp] = part;
         if (++kg == kUnitGroup && g + tm.G < NG) {
           flush(part_r, u0, kg);
           kg = 0;
@@ -410,12 +471,8 @@ __device__ bool cg_cells(const DevPlan& P, Team& tm, unsigned char* dsm, double 
       }
       if (!phase_end<NW>(tm, wpart, part_r, u0, kg)) return false;
     }
-    // ================= phase 2: t = sum over groups; p, z, x, s of the owned chunk
+    // ================= phase 2: t = sum over groups; s, p, x of the owned chunk
     {
-      // gamma's partials alternate: a block may finish this phase while another
-      // still reads the previous ones
-      const float2* const pc_in = part_c + ((it & 1) ? nown : 0);
-      float2* const pc_out = part_c + ((it & 1) ? 0 : nown);
       const int mi = tid % CW, gl = tid / CW;
       auto sum_t = [&](int m) -> float {
         float a = 0.0f;
@@ -432,7 +489,7 @@ __device__ bool cg_cells(const DevPlan& P, Team& tm, unsigned char* dsm, double 
       };
       float* const comb = reinterpret_cast<float*>(dsm);  // [LG][CW] when LG > 1
       int c = tm.rank;
-      float t = 0.0f, so = 0.0f, po = 0.0f, zo = 0.0f, xo = 0.0f;
+      float t = 0.0f, so = 0.0f, po = 0.0f, xo = 0.0f;
       auto load = [&](int ch) {
         const int m = ch * CW + mi;
         t = 0.0f;
@@ -440,52 +497,20 @@ __device__ bool cg_cells(const DevPlan& P, Team& tm, unsigned char* dsm, double 
           if (gl == 0) {
             so = ldcg(sv + m);
             xo = ldcg(xv + m);
-            if (it > 0) {
-              po = ldcg(pv + m);
-              zo = ldcg(zv + m);
-            }
+            if (!first) po = ldcg(pv + m);
           }
           t = sum_t(m);
         }
       };
       if (warp == 0) {
-        float2 gs, dl;
-        warp0_sum2(pc_in, it > 0 ? nown : 0, part_r, NG, &gs, &dl);
+        const float2 dl = warp0_sum(part_r, NG);
         if (tid == 0) {
-          if (it > 0) gam = gs;
           int cc = 0;
-          float2 al = make_float2(0.0f, 0.0f), bt = al;
-          if (!isfinite(gam.x) || !isfinite(dl.x)) {
-            cc = FCT_ERR_NONFINITE + 16;
-          } else if (it > 0 && gam.x <= tol2) {
-            cc = 1;
-          } else if (it >= max_iter) {
-            cc = FCT_ERR_NOCONV + 16;
-          } else if (it > 0 && stall > 0) {
-            if (gam.x < best) {
-              best = gam.x;
-              best_it = it;
-            } else if (it - best_it >= stall) {
-              cc = 1;
-            }
-          }
-          if (cc == 0) {
-            float2 den = dl;
-            if (it > 0) {
-              bt = df_div(gam, gam_prev);
-              const float2 u = df_div(df_mul(bt, gam), al_prev);
-              den = df_add(dl, make_float2(-u.x, -u.y));
-            }
-            if (!(den.x > 0.0f)) {
-              cc = 1;  // no further progress in this precision
-            } else {
-              al = df_div(gam, den);
-              gam_prev = gam;
-              al_prev = al;
-            }
-          }
-          sh_ab[0] = al.x;
-          sh_ab[1] = bt.x;
+          float al = 0.0f;
+          if (!isfinite(dl.x)) cc = FCT_ERR_NONFINITE + 16;
+          else if (!(dl.x > 0.0f)) cc = 1;  // q = 0: s is already zero to working precision
+          else al = df_div(gam, dl).x;
+          sh_ab[0] = al;
           sh_ctl[0] = cc;
         }
       }
@@ -507,26 +532,26 @@ __device__ bool cg_cells(const DevPlan& P, Team& tm, unsigned char* dsm, double 
         const int m = c * CW + mi;
         float2 part = make_float2(0.0f, 0.0f);
         if (gl == 0 && m < N) {
-          const float pn = it > 0 ? fmaf(beta, po, so) : so;
-          const float zn = it > 0 ? fmaf(beta, zo, t) : t;
-          const float sn = fmaf(-alpha, zn, so);
+          const float pn = first ? so : fmaf(beta, po, so);
+          const float sn = fmaf(-alpha, t, so);
           stcg(sv + m, sn);
           stcg(pv + m, pn);
-          stcg(zv + m, zn);
           stcg(xv + m, fmaf(alpha, pn, xo));
           part = df_square(sn * rsf);
         }
         part = warp_sum(part);
-        if ((tid & 31) == 0) wpart[kg][warp] = part;
+        if (lane == 0) wpart[kg][warp] = part;
         if (++kg == kUnitGroup && c + tm.G < nown) {
-          flush(pc_out, u0, kg);
+          flush(part_c, u0, kg);
           kg = 0;
           u0 = c + tm.G;
         }
       }
-      if (!phase_end<NW>(tm, wpart, pc_out, u0, kg)) return false;
+      if (!phase_end<NW>(tm, wpart, part_c, u0, kg)) return false;
     }
+    first = false;
   }
+  team.epoch = tm.epoch;
   if (tid == 0) {
     sh_ctl[1] = ctl >= 16 ? ctl - 16 : FCT_OK;
     sh_ctl[2] = it;

@@ -146,6 +146,26 @@ __device__ __forceinline__ float2 df_square(float t) {
   const float hi = __fmul_rn(t, t);  // not contracted into the sum that follows
   return make_float2(hi, fmaf(t, t, -hi));
 }
+// Products and quotients of pairs (about 44 bits), for the scalars of the FP32
+// inner solves.
+__device__ __forceinline__ float2 df_mul(float2 a, float2 b) {
+  const float p = __fmul_rn(a.x, b.x);
+  const float e = fmaf(a.x, b.x, -p) + fmaf(a.x, b.y, __fmul_rn(a.y, b.x));
+  const float hi = p + e;
+  return make_float2(hi, e - (hi - p));
+}
+__device__ __forceinline__ float2 df_div(float2 a, float2 b) {
+  const float q1 = __fdividef(a.x, b.x);
+  const float2 qb = df_mul(make_float2(q1, 0.0f), b);
+  const float2 r = df_add(a, make_float2(-qb.x, -qb.y));
+  const float q2 = __fdividef(r.x, b.x);
+  const float hi = q1 + q2;
+  return make_float2(hi, q2 - (hi - q1));
+}
+__device__ __forceinline__ float2 df_of(double v) {
+  const float hi = static_cast<float>(v);
+  return make_float2(hi, static_cast<float>(v - static_cast<double>(hi)));
+}
 __device__ __forceinline__ float2 warp_sum(float2 v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1)
@@ -184,6 +204,20 @@ __device__ __forceinline__ float2 pzero_part(float2) { return make_float2(0.0f, 
 __device__ __forceinline__ float2 padd(float2 a, float2 b) { return df_add(a, b); }
 __device__ __forceinline__ float2 pzero(float2) { return make_float2(0.0f, 0.0f); }
 
+// Sum of a unit's NW per-warp partials: a tree over values loaded side by side
+// (a chain of NW dependent additions is on the path to every team barrier).
+template <int NW, typename PT>
+__device__ __forceinline__ PT warps_sum(const PT (&w)[NW]) {
+  PT v[NW];
+#pragma unroll
+  for (int i = 0; i < NW; ++i) v[i] = w[i];
+#pragma unroll
+  for (int s = 1; s < NW; s <<= 1)
+#pragma unroll
+    for (int i = 0; i + s < NW; i += 2 * s) v[i] = padd(v[i], v[i + s]);
+  return v[0];
+}
+
 template <int NW, typename PT>
 __device__ bool phase_end(Team& tm, const PT (*wpart)[NW], PT* part, int u0, int nk) {
   __shared__ int s_ok2;
@@ -191,10 +225,7 @@ __device__ bool phase_end(Team& tm, const PT (*wpart)[NW], PT* part, int u0, int
   tm.epoch += 1;
   if (threadIdx.x < 32) {
     if (static_cast<int>(threadIdx.x) < nk) {
-      PT v = pzero(PT{});
-#pragma unroll
-      for (int w = 0; w < NW; ++w) v = padd(v, wpart[threadIdx.x][w]);
-      stcg(part + u0 + static_cast<int>(threadIdx.x) * tm.G, v);
+      stcg(part + u0 + static_cast<int>(threadIdx.x) * tm.G, warps_sum<NW>(wpart[threadIdx.x]));
     }
     __syncwarp();
     if (threadIdx.x == 0) {
@@ -261,8 +292,7 @@ __device__ __forceinline__ double warp0_sum(const double* part, int n) {
     for (int j = 0; j < 8; ++j) t[j] = ldcg(part + min(i0 + 32 * j, n - 1));  // every load issued
 #pragma unroll
     for (int j = 0; j < 8; ++j) t[j] = i0 + 32 * j < n ? t[j] : 0.0;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) v += t[j];
+    v += ((t[0] + t[1]) + (t[2] + t[3])) + ((t[4] + t[5]) + (t[6] + t[7]));
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -271,9 +301,8 @@ __device__ __forceinline__ double warp0_sum(const double* part, int n) {
 
 // Warp 0: double-float sum of n per-unit partials (hi, lo) in a fixed order,
 // on the FP32 pipe: 8 independent accumulators per lane (one per load slot of
-// a round) keep the dependent chain short; the result (every lane) is the
-// pair's FP64 value.
-__device__ __forceinline__ double warp0_sum(const float2* part, int n) {
+// a round) keep the dependent chain short; every lane gets the pair.
+__device__ __forceinline__ float2 warp0_sum(const float2* part, int n) {
   float2 acc[8];
 #pragma unroll
   for (int j = 0; j < 8; ++j) acc[j] = make_float2(0.0f, 0.0f);
@@ -288,7 +317,7 @@ __device__ __forceinline__ double warp0_sum(const float2* part, int n) {
   }
   const float2 s = df_add(df_add(df_add(acc[0], acc[1]), df_add(acc[2], acc[3])),
                           df_add(df_add(acc[4], acc[5]), df_add(acc[6], acc[7])));
-  return widen(warp_sum(s));
+  return warp_sum(s);
 }
 
 // Warp 0: FP64 pair sums of n partials in a fixed order (lane 0 holds the result).

@@ -433,20 +433,21 @@ CellBytes cell_bytes(const CellLayout& L, int K) {
   b.dest = sizeof(uint16_t) * cells * L.gmax * 32;
   b.wtab = sizeof(int2) * cells * (L.warps + 1);
   b.comb = sizeof(int2) * cells * L.cmax;
-  b.ncomb = sizeof(int32_t) * cells;
+  b.ncomb = sizeof(int2) * cells;
   return b;
 }
 
 // Layout of the mixed path's inner solve by grid groups for a plan with
 // L->rows filled in.
-fct_status choose_cell_layout(fct_plan P, int64_t R, int64_t wave, CellLayout* L) {
+fct_status choose_cell_layout(fct_plan P, int64_t wave, CellLayout* L) {
+  if (!cells_pay(P->N, P->K, P->block_threads, wave)) return FCT_OK;  // before the device is asked
   int dev = 0, cap = 0, per_sm = 0;
   FCT_CUDA(cudaGetDevice(&dev));
   cudaDeviceProp prop;
   FCT_CUDA(cudaGetDeviceProperties(&prop, dev));
   const fct_status s = solver_smem_cap(P->block_threads, prop, &cap, &per_sm);
   if (s != FCT_OK) return s;
-  choose_cells(P->N, R, P->K, P->M, P->block_threads, wave, cap, L);
+  choose_cells(P->N, P->K, P->M, P->block_threads, wave, cap, L);
   return FCT_OK;
 }
 
@@ -653,7 +654,7 @@ fct_status fct_plan_create(fct_plan* out, int D, int64_t N, const uint16_t* supp
     if (o.precision == FCT_MIXED) {
       CL.rows.resize(K);
       for (int l = 0; l < K; ++l) CL.rows[l] = H.row_off[l + 1] - H.row_off[l];
-      s = choose_cell_layout(P, H.R, wave, &CL);
+      s = choose_cell_layout(P, wave, &CL);
       if (s != FCT_OK) {
         delete P;
         return s;
@@ -682,7 +683,7 @@ fct_status fct_plan_create(fct_plan* out, int D, int64_t N, const uint16_t* supp
   }
   if (on_device && o.precision == FCT_MIXED) {
     CL.rows = DT.grid_rows;
-    s = choose_cell_layout(P, H.R, wave, &CL);
+    s = choose_cell_layout(P, wave, &CL);
     if (s != FCT_OK) {
       delete P;
       return s;

@@ -246,7 +246,7 @@ struct DevPlan {
   const uint16_t* tk_dest;   // [cells][tk_gmax][32] where a run's sum goes: row, or extra slot
   const int2* tk_wtab;       // [cells][warps + 1] first block and first group of each warp
   const int2* tk_comb;       // [cells][tk_cmax] rows of several runs: row | runs << 16, first extra slot
-  const int32_t* tk_ncomb;   // [cells]
+  const int2* tk_ncomb;      // [cells] rows of more than kCellFew runs (from the start), of fewer (from the end)
   const int32_t* tk_rows;    // [K] rows of the grid
   const int32_t* tk_qoff;    // [K] start of the grid's row sums inside its group's
 };
@@ -426,12 +426,23 @@ struct CellLayout {
   int32_t q = 0, ext = 0, blocks = 0, gmax = 0, cmax = 0, cw = 0, lg = 0, nown = 0, smem = 0;
   std::vector<int32_t> rows, qoff;  // [K]
 };
-constexpr int kCellRun = 32;          // longest run of a row
+// The plans that take it: at least as many grids as SMs (`wave` co-resident blocks;
+// with fewer, SMs idle: D = 10 degree 8, 30 grids: 34 us per CG iteration against
+// 18 in the two-matrix form), and enough coefficients and entries that the work
+// outweighs its phases' longer latency (D = 60, N = 5027, 637 grids: 48 us against
+// 39; D = 30, N = 6371, 202 grids: 30 against 42; D = 100, N = 50000, 240 grids:
+// 72 against 226).
+constexpr int64_t kCellMinN = 6144;
+constexpr int64_t kCellMinEntries = int64_t{1} << 20;
+bool cells_pay(int64_t N, int K, int block_threads, int64_t wave);
+constexpr int kCellRun = 64;          // longest run of a row
+constexpr int kCellIdle = 5;          // idle groups after a cell's last (destinations read ahead)
+constexpr int kCellFew = 8;           // runs of a row that one thread adds up
 constexpr int kCellMaxSlice = 32736;  // 15-bit coefficient index, 32 padding slots included
 // Chooses the layout from the rows of every grid (L->rows), the block size,
 // the co-resident blocks `wave`, the shared memory `cap` a block may take and
 // the M doubles of each DCT buffer.  groups stays 0 where it does not fit.
-void choose_cells(int64_t N, int64_t R, int K, int64_t M, int block_threads, int64_t wave, int cap, CellLayout* L);
+void choose_cells(int64_t N, int K, int64_t M, int block_threads, int64_t wave, int cap, CellLayout* L);
 // Cell tables (see DevPlan).  The device build takes the build's pre-order
 // tables and is ordered on its stream; the host build takes H before
 // device_row_order and fills host arrays of the same sizes.  Both give the
@@ -440,8 +451,7 @@ struct CellPointers {
   uint16_t* idx;
   float* w;
   uint16_t* dest;
-  int2 *wtab, *comb;
-  int32_t* ncomb;
+  int2 *wtab, *comb, *ncomb;
 };
 fct_status build_cells_device(const DeviceTables& T, int64_t N, int K, const CellLayout& L, const CellPointers& out);
 void build_cells_host(const HostTables& H, const CellLayout& L, const CellPointers& out);

@@ -576,9 +576,9 @@ __global__ void __launch_bounds__(kScanThreads) cell_build_kernel(const CellArgs
     idx[i] = static_cast<uint16_t>(a.SL + ((i >> 2) & 31));
     wv[i] = 0.0f;
   }
-  for (int i = t; i < min(G + 2, a.gmax) * 32; i += kScanThreads) dest[i] = static_cast<uint16_t>(nrow + a.ext);
+  for (int i = t; i < min(G + kCellIdle, a.gmax) * 32; i += kScanThreads) dest[i] = static_cast<uint16_t>(nrow + a.ext);
   // 4. places of the rows' last runs; cut rows
-  int32_t next = 0, ncomb = 0;
+  int32_t next = 0, many = 0, few = 0;
   for (int i0 = 0; i0 < nslot; i0 += kScanThreads) {
     const int i = i0 + t;
     int32_t len = 0, nf = 0, tail = 0;
@@ -605,18 +605,21 @@ __global__ void __launch_bounds__(kScanThreads) cell_build_kernel(const CellArgs
     if (i < nslot) rlast[i] = base[tail] + wcnt[warp][tail] + __popc(peers & ((1u << lane) - 1u));
     const int32_t e = next + block_exclusive_scan(nf > 0 ? nf + 1 : 0, &total);
     next += total;
-    const int32_t ci = ncomb + block_exclusive_scan(nf > 0 ? 1 : 0, &total);
-    ncomb += total;
+    const bool is_many = nf + 1 > kCellFew, is_few = nf > 0 && !is_many;
+    const int32_t cm = many + block_exclusive_scan(is_many ? 1 : 0, &total);
+    many += total;
+    const int32_t cf = few + block_exclusive_scan(is_few ? 1 : 0, &total);
+    few += total;
     if (i < nslot) {
       const int32_t row = static_cast<int32_t>(ent[start[i]] >> 16);
       if (nf > 0) {
-        a.out.comb[cell * a.cmax + ci] = make_int2(row | ((nf + 1) << 16), nrow + e);
+        a.out.comb[cell * a.cmax + (is_many ? cm : a.cmax - 1 - cf)] = make_int2(row | ((nf + 1) << 16), nrow + e);
         for (int k = 0; k < nf; ++k) dest[rfull[i] + k] = static_cast<uint16_t>(nrow + e + k);
       }
       dest[rlast[i]] = static_cast<uint16_t>(nf > 0 ? nrow + e + nf : row);
     }
   }
-  if (t == 0) a.out.ncomb[cell] = ncomb;
+  if (t == 0) a.out.ncomb[cell] = make_int2(many, few);
   __syncthreads();
   // 5. entries
   auto place = [&](int32_t rank, int k) {

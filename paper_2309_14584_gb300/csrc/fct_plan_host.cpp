@@ -544,26 +544,28 @@ void normal_matrix(const HostTables& H, std::vector<int32_t>* rowptr, std::vecto
   }
 }
 
-void choose_cells(int64_t N, int64_t R, int K, int64_t M, int block_threads, int64_t wave, int cap, CellLayout* L) {
+bool cells_pay(int64_t N, int K, int block_threads, int64_t wave) {
+  return K >= wave * block_threads / 512 && N >= kCellMinN && K * N >= kCellMinEntries;
+}
+
+void choose_cells(int64_t N, int K, int64_t M, int block_threads, int64_t wave, int cap, CellLayout* L) {
   L->groups = 0;
-  if (wave < 1) wave = 1;
-  if (R < N) return;  // rank-deficient; the solver keeps an N-vector in the row workspace
   L->qoff.assign(K, 0);
   L->warps = block_threads / 32;
   const int64_t ncap = (N + 31) / 32 * 32;
   // one task per co-resident block: as many grids per group as that takes;
   // fewer where a group's row sums leave no room for a slice
   for (int gg = static_cast<int>((K + wave - 1) / wave); gg >= 1; gg = gg > 1 ? gg / 2 : 0) {
-    // the slice and the extra slots (2 per kCellRun coefficients and grid)
-    // share the room the rows leave
+    // the slice and the extra slots (2 per kCellRun coefficients and grid, with
+    // their destinations) share the room the rows leave
     int64_t rmax = 0;
     for (int l0 = 0; l0 < K; l0 += gg) {
       int64_t q = 0;
-      for (int l = l0; l < std::min(K, l0 + gg); ++l) q += (3 * L->rows[l]) / 2 + 72;
+      for (int l = l0; l < std::min(K, l0 + gg); ++l) q += (3 * L->rows[l]) / 2 + 120;
       rmax = std::max(rmax, q);
     }
     const int64_t room = cap / 4 - rmax - 64;
-    int64_t sl = room * 64 / (64 + 6 * gg);
+    int64_t sl = room * kCellRun / (kCellRun + 3 * gg);
     sl = std::min({sl, ncap, static_cast<int64_t>(kCellMaxSlice)}) / 32 * 32;
     if (sl < std::min<int64_t>(ncap, 2048)) continue;
     const int64_t S = (N + sl - 1) / sl;
@@ -578,8 +580,8 @@ void choose_cells(int64_t N, int64_t R, int K, int64_t M, int block_threads, int
       for (int l = l0; l < std::min(K, l0 + gg); ++l) {
         L->qoff[l] = static_cast<int32_t>(q);
         // row sums, then the run destinations (16 bits; up to 31 idle lanes in
-        // the last group and two groups after it)
-        q += (L->rows[l] + ext + 1 + 3) / 4 * 4 + ((L->rows[l] + ext + 31) / 32 + 2) * 16;
+        // the last group and kCellIdle groups after it)
+        q += (L->rows[l] + ext + 1 + 3) / 4 * 4 + ((L->rows[l] + ext + 31) / 32 + kCellIdle) * 16;
         fits = fits && L->rows[l] + ext + 1 <= 65535;
       }
       qmax = std::max(qmax, q);
@@ -601,7 +603,7 @@ void choose_cells(int64_t N, int64_t R, int K, int64_t M, int block_threads, int
     // sorted by length, 32 to a group, padding is at most kCellRun steps; each
     // warp's share is padded to four
     L->blocks = static_cast<int32_t>((sl / 32 + kCellRun + 1 + 3 * L->warps + 3) / 4 + 1);
-    L->gmax = static_cast<int32_t>(sl / 32 + 3);
+    L->gmax = static_cast<int32_t>(sl / 32 + 1 + kCellIdle);
     L->cmax = static_cast<int32_t>(sl / kCellRun + 1);
     L->cw = static_cast<int32_t>(cw);
     L->lg = static_cast<int32_t>(block_threads / cw);
@@ -629,7 +631,7 @@ void build_cells_host(const HostTables& H, const CellLayout& L, const CellPointe
       auto row_of = [&](int j) { return H.crow[l * N + c[j]] - r0; };
       // runs by length: the full runs of long rows first, then every row's last
       std::vector<std::vector<Run>> full(kCellRun + 1), last(kCellRun + 1);
-      int32_t ext = 0, ncomb = 0;
+      int32_t ext = 0, many = 0, few = 0;
       for (int j = 0; j < n;) {
         int e = j;
         while (e < n && row_of(e) == row_of(j)) ++e;
@@ -638,12 +640,13 @@ void build_cells_host(const HostTables& H, const CellLayout& L, const CellPointe
         const int tail = len - nf * kCellRun;
         last[tail].push_back({j + nf * kCellRun, tail, nf > 0 ? nrow + ext + nf : row_of(j)});
         if (nf > 0) {
-          o.comb[cell * L.cmax + ncomb++] = int2{row_of(j) | ((nf + 1) << 16), nrow + ext};
+          o.comb[cell * L.cmax + (nf + 1 > kCellFew ? many++ : L.cmax - 1 - few++)] =
+              int2{row_of(j) | ((nf + 1) << 16), nrow + ext};
           ext += nf + 1;
         }
         j = e;
       }
-      o.ncomb[cell] = ncomb;
+      o.ncomb[cell] = int2{many, few};
       std::vector<Run> runs;
       for (int k = kCellRun; k >= 1; --k) {
         runs.insert(runs.end(), full[k].begin(), full[k].end());
@@ -669,7 +672,7 @@ void build_cells_host(const HostTables& H, const CellLayout& L, const CellPointe
           idx[b * 128 + i] = static_cast<uint16_t>(SL + i / 4);
           wv[b * 128 + i] = 0.0f;
         }
-      for (int i = 0; i < std::min(G + 2, L.gmax) * 32; ++i) dest[i] = static_cast<uint16_t>(nrow + L.ext);
+      for (int i = 0; i < std::min(G + kCellIdle, L.gmax) * 32; ++i) dest[i] = static_cast<uint16_t>(nrow + L.ext);
       for (int w = 0; w < NW; ++w)
         for (int g = gb[w]; g < gb[w + 1]; ++g)
           for (int k = 0; k < off[g + 1] - off[g]; ++k) {

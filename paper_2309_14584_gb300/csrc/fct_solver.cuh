@@ -618,6 +618,20 @@ __device__ __forceinline__ bool coef_owner(const DevPlan& P, int c, int wk, int*
 // ---------------------------------------------------------------------------
 constexpr int kUnitGroup = 16;  // units per flush of the per-warp partials
 
+// The scalars behind alpha and beta, computed by one thread between two team
+// barriers of every phase: in FP64 for FP64 vectors, as double-float pairs on the
+// FP32 pipe for FP32 vectors (GB300's FP64 units are far apart: an FP64 quotient
+// on this path took longer than a whole gather of a small plan).
+__device__ __forceinline__ bool sc_finite(double v) { return isfinite(v); }
+__device__ __forceinline__ bool sc_finite(float2 v) { return isfinite(v.x); }
+__device__ __forceinline__ double sc_val(double v) { return v; }
+__device__ __forceinline__ float sc_val(float2 v) { return v.x; }
+__device__ __forceinline__ double sc_div(double a, double b) { return a / b; }
+__device__ __forceinline__ float sc_div(float2 a, float2 b) { return df_div(a, b).x; }
+template <typename PT> __device__ __forceinline__ PT sc_of(double v);
+template <> __device__ __forceinline__ double sc_of<double>(double v) { return v; }
+template <> __device__ __forceinline__ float2 sc_of<float2>(double v) { return df_of(v); }
+
 #include "fct_cells.cuh"
 
 template <int BT, typename V, typename WT, typename XT, bool SV, int DEEP>
@@ -628,7 +642,8 @@ __device__ bool cg_normal(const DevPlan& P, Team& tm, const BlockTabs& T, const 
   using PT = typename SqPart<V>::T;
   constexpr int NW = BT / 32 - 1;  // worker warps
   __shared__ PT wpart[kUnitGroup][NW];
-  __shared__ double sh_ab[2];      // beta, alpha
+  __shared__ V sh_ab[2];           // beta, alpha
+  __shared__ double sh_gam;
   __shared__ int sh_ctl[3];        // stop flag, status, iterations
   *status_out = FCT_OK;
   *iters_out = 0;
@@ -645,9 +660,10 @@ __device__ bool cg_normal(const DevPlan& P, Team& tm, const BlockTabs& T, const 
   frexp(gamma0, &e0);
   const double rs = ldexp(1.0, -(e0 / 2));  // power of two near 1/sqrt(gamma0): exact scaling
   const double c0 = gamma0 * rs * rs;       // gamma0 in scaled units (in [1/4, 4))
-  const double tol2 = tol * tol * c0;
+  const V tol2 = static_cast<V>(tol * tol * c0);
   // thread 0's state (scaled gamma)
-  double gam = c0, best = c0;
+  PT gam = sc_of<PT>(c0);
+  V best = sc_val(gam);
   int it = 0, best_it = 0;
   bool first = true;
   // lead lanes of a unit sit at multiples of its lanes per row (coefficient)
@@ -666,10 +682,7 @@ __device__ bool cg_normal(const DevPlan& P, Team& tm, const BlockTabs& T, const 
   auto flush = [&](PT* part, int u0, int nk) {
     __syncthreads();
     if (threadIdx.x < nk) {
-      PT v = pzero(PT{});
-#pragma unroll
-      for (int w2 = 0; w2 < NW; ++w2) v = padd(v, wpart[threadIdx.x][w2]);
-      stcg(part + u0 + threadIdx.x * tm.G, v);
+      stcg(part + u0 + threadIdx.x * tm.G, warps_sum<NW>(wpart[threadIdx.x]));
     }
     __syncthreads();
   };
@@ -687,23 +700,23 @@ __device__ bool cg_normal(const DevPlan& P, Team& tm, const BlockTabs& T, const 
       if (wk >= 0) {
         if (u < nru) gather_a(u, 0, &as, &ap, &row, &lead);
       } else {
-        double gnew = 1.0;
-        if (!first) gnew = widen(warp0_sum(part_c, ncc));
+        PT gnew = gam;
+        if (!first) gnew = warp0_sum(part_c, ncc);
         if (threadIdx.x == 0) {
           int c = 0;
-          double bt = 0.0;
+          V bt = V(0);
           if (!first) {
             ++it;
-            if (!isfinite(gnew)) {
+            if (!sc_finite(gnew)) {
               c = FCT_ERR_NONFINITE + 16;
             } else {
-              bt = gnew / gam;
+              bt = sc_div(gnew, gam);
               gam = gnew;
-              if (gam <= tol2) c = 1;
+              if (sc_val(gam) <= tol2) c = 1;
               else if (it >= max_iter) c = FCT_ERR_NOCONV + 16;
               else if (stall > 0) {
-                if (gam < best) {
-                  best = gam;
+                if (sc_val(gam) < best) {
+                  best = sc_val(gam);
                   best_it = it;
                 } else if (it - best_it >= stall) {
                   c = 1;
@@ -718,7 +731,7 @@ __device__ bool cg_normal(const DevPlan& P, Team& tm, const BlockTabs& T, const 
       __syncthreads();
       ctl = sh_ctl[0];
       if (ctl != 0) break;
-      const V beta = static_cast<V>(sh_ab[0]);
+      const V beta = sh_ab[0];
       int k = 0, kg = 0, u0 = u;
       for (; u < nru; u += tm.G, ++k) {
         if (k > 0 && wk >= 0) gather_a(u, k, &as, &ap, &row, &lead);
@@ -760,24 +773,23 @@ __device__ bool cg_normal(const DevPlan& P, Team& tm, const BlockTabs& T, const 
           t = coef_gather<V, WT, SV, (8 << DEEP)>(P, T, wcm, c, 0, wk, &m, &lead, [&](int i) { return q[i]; });
         }
       } else {
-        const double dl = widen(warp0_sum(part_r, nru));
+        const PT dl = warp0_sum(part_r, nru);
         if (threadIdx.x == 0) {
           int cc = 0;
-          double al = 0.0;
-          if (!isfinite(dl)) cc = FCT_ERR_NONFINITE + 16;
-          else if (!(dl > 0.0)) cc = 1;  // q = 0: s is already zero to working precision
-          else al = gam / dl;
+          V al = V(0);
+          if (!sc_finite(dl)) cc = FCT_ERR_NONFINITE + 16;
+          else if (!(sc_val(dl) > V(0))) cc = 1;  // q = 0: s is already zero to working precision
+          else al = sc_div(gam, dl);
           sh_ab[1] = al;
           sh_ctl[0] = cc;
           if (P.hist != nullptr && tm.rank == 0 && cc == 0 && pass < P.hist_cap)
-            P.hist[pass] = make_double2(al, first ? 0.0 : sh_ab[0]);
+            P.hist[pass] = make_double2(al, first ? 0.0 : static_cast<double>(sh_ab[0]));
         }
       }
       __syncthreads();
       ctl = sh_ctl[0];
       if (ctl != 0) break;
-      const V alpha = static_cast<V>(sh_ab[1]);
-      const V beta = static_cast<V>(sh_ab[0]);
+      const V alpha = sh_ab[1], beta = sh_ab[0];
       int k = 0, kg = 0, c0 = c;
       for (; c < ncc; c += tm.G, ++k) {
         if (k > 0 && wk >= 0) {
@@ -811,12 +823,12 @@ __device__ bool cg_normal(const DevPlan& P, Team& tm, const BlockTabs& T, const 
   if (threadIdx.x == 0) {
     sh_ctl[1] = ctl >= 16 ? ctl - 16 : FCT_OK;
     sh_ctl[2] = it;
-    sh_ab[0] = gam;
+    sh_gam = widen(gam);
   }
   __syncthreads();
   *status_out = sh_ctl[1];
   *iters_out = sh_ctl[2];
-  *gamma_out = sh_ab[0] / (rs * rs);
+  *gamma_out = sh_gam / (rs * rs);
   __syncthreads();
   return true;
 }
@@ -916,10 +928,7 @@ __device__ bool pcg_normal_w(const DevPlan& P, Team& tm, const BlockTabs& T, dou
   auto flush2 = [&](double2* part, int u0, int nk) {
     __syncthreads();
     if (threadIdx.x < nk) {
-      double2 v = make_double2(0.0, 0.0);
-#pragma unroll
-      for (int w2 = 0; w2 < NW; ++w2) v = padd(v, wpart2[threadIdx.x][w2]);
-      stcg(part + u0 + threadIdx.x * tm.G, v);
+      stcg(part + u0 + threadIdx.x * tm.G, warps_sum<NW>(wpart2[threadIdx.x]));
     }
     __syncthreads();
   };
@@ -1075,7 +1084,21 @@ __device__ bool pcg_normal_w(const DevPlan& P, Team& tm, const BlockTabs& T, dou
 // ---------------------------------------------------------------------------
 template <int BT, bool SV, int DEEP>
 __device__ bool solve_job(const SolveJob& J, Team& tm, double* red, unsigned char* dsm, int smem_bytes) {
-  const DevPlan& P = *J.plan;
+  // The plan's header in shared memory: every barrier's gpu-scope acquire drops
+  // L1, so the first use after a barrier of a field held in global memory would
+  // cost an L2 round trip, and a phase starts with a chain of them (D = 6 degree
+  // 10: 7.0 -> 6.8 us per CG iteration).
+  __shared__ DevPlan sP;
+  {
+    static_assert(sizeof(DevPlan) % 8 == 0, "DevPlan is copied in 8-byte words");
+    __syncthreads();  // the previous job's readers are done
+    const unsigned long long* src = reinterpret_cast<const unsigned long long*>(J.plan);
+    for (int i = threadIdx.x; i < static_cast<int>(sizeof(DevPlan) / 8); i += BT)
+      reinterpret_cast<unsigned long long*>(&sP)[i] = src[i];
+    __syncthreads();
+  }
+  const DevPlan& P = sP;
+  BlockTabs T;
   if (P.coef_split && smem_bytes < coef_combine_bytes(BT)) {  // the host sizes launches to hold them
     if (threadIdx.x == 0) atomicExch(tm.err, static_cast<int>(FCT_ERR_INVALID_ARG));
     return false;
@@ -1087,7 +1110,6 @@ __device__ bool solve_job(const SolveJob& J, Team& tm, double* red, unsigned cha
     if (threadIdx.x == 0) atomicExch(tm.err, static_cast<int>(FCT_ERR_INVALID_ARG));
     return false;
   }
-  BlockTabs T;
   load_block_tabs<BT>(P, tm, dsm, smem_bytes, &T, J.precision == FCT_MIXED && P.n_w_units > 0 && P.s_init == nullptr,
                       SV ? (J.precision == FCT_MIXED ? 4 : 8) : 0, !cells);
   const int ncc = P.n_coef_chunks, nre = P.n_rowel_chunks, nru = P.n_row_units, nwide = P.n_wide_units;
