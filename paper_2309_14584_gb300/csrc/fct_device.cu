@@ -1322,9 +1322,37 @@ static fct_status batch_setup(int B, const fct_plan* plans, const double* const*
   }
   int G = team_blocks;
   if (G <= 0) {
-    int units = 0;
-    for (int i = 0; i < B; ++i) units = std::max(units, plans[i]->grid_blocks);
-    G = std::max(1, std::min(units, P0->max_coresident / std::max(1, std::min(B, 16))));
+    // Blocks per team from a model of the launch: a CG iteration of a transform
+    // takes kIterUs of latency plus its entries over the team's threads (fitted to
+    // D = 10 degree 8 on 38..304 blocks: 18.5, 50, 101 us against 18.6, 55, 102),
+    // the jobs go to the teams largest first, and the last team to finish counts.
+    // A fixed share of the GPU per job leaves most of it idle once only the
+    // largest transforms of an unlike batch are left.
+    constexpr double kIterUs = 6.5, kEntryUs = 0.717;
+    std::vector<double> work(B);
+    int units = 1;
+    for (int q = 0; q < B; ++q) {
+      const fct_plan Pq = plans[order[q]];
+      work[q] = kEntryUs * static_cast<double>(Pq->hp.K) * static_cast<double>(Pq->N) / P0->block_threads *
+                (Pq->opt.precision == FCT_MIXED ? 1.0 : 2.0);
+      units = std::max(units, Pq->grid_blocks);
+    }
+    double best = 0.0;
+    std::vector<double> busy;
+    int last = 0;
+    for (int teams = 1; teams <= std::min({B, kMaxTeams, P0->max_coresident}); teams = teams < 8 ? teams + 1 : teams * 5 / 4) {
+      const int g = std::min(units, P0->max_coresident / teams);
+      if (g == last) continue;
+      last = g;
+      busy.assign(std::min(P0->max_coresident / g, std::min(B, kMaxTeams)), 0.0);
+      for (int q = 0; q < B; ++q)
+        *std::min_element(busy.begin(), busy.end()) += kIterUs + work[q] / g;
+      const double t = *std::max_element(busy.begin(), busy.end());
+      if (G <= 0 || t < best) {
+        best = t;
+        G = g;
+      }
+    }
   }
   G = std::min(G, P0->max_coresident);
   *teams_out = std::min(std::max(1, P0->max_coresident / G), std::min(B, kMaxTeams));
