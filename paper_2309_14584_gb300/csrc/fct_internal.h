@@ -456,6 +456,15 @@ struct CellPointers {
 fct_status build_cells_device(const DeviceTables& T, int64_t N, int K, const CellLayout& L, const CellPointers& out);
 void build_cells_host(const HostTables& H, const CellLayout& L, const CellPointers& out);
 
+// Evaluation program of a support (eval_trie_kernel): its terms in `chunks`
+// programs of consecutive terms, chunk c starting at word[c] (word[chunks] = the
+// end, word[chunks + 1] = the most nonzero components of an index).  tk = table
+// entries per axis.  prog holds at most (nonzero components) + N + chunks x D
+// words; scratch: 16 N bytes, at least 256.  Ordered on `stream`.
+inline int eval_chunks(int64_t N) { return N < 32 ? 1 : (N >= 1024 ? 64 : static_cast<int>(N / 16)); }
+fct_status build_eval_program(const uint16_t* d_support, int64_t N, int D, int tk, int chunks, uint32_t* prog,
+                              int32_t* word, void* scratch, void* stream);
+
 // W = A^T A (N x N, CSR, columns ascending, FP64 sums in a fixed order) and
 // the bound sum over rows of A of (row length)^2 >= nnz(W), cheap to compute
 // before deciding to build W.

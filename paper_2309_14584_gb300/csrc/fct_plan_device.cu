@@ -651,6 +651,61 @@ __global__ void __launch_bounds__(kScanThreads) cell_build_kernel(const CellArgs
 
 __global__ void set_int_kernel(int32_t* dst, int32_t v) { *dst = v; }
 
+// Evaluation program (see eval_trie_kernel).  Term m of chunk c = m's chunk: words
+// that close the previous term's nodes beyond the common prefix (none at a chunk's
+// start), one word with the nodes it opens, and at a chunk's end words that close
+// its own.  fill = false: cnt[m] = the number of words (cnt[N] = 0).
+__global__ void eval_words_kernel(int64_t N, int D, int tk, int chunks, const uint16_t* __restrict__ support,
+                                  bool fill, int32_t* __restrict__ cnt, uint32_t* __restrict__ prog,
+                                  int32_t* __restrict__ word) {
+  __shared__ int s_most;
+  int most = 0;  // nonzero components of an index
+  if (threadIdx.x == 0) s_most = 0;
+  __syncthreads();
+  for (int64_t m = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; m <= N;
+       m += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+    if (m == N) {
+      if (fill) word[chunks] = cnt[N];
+      else cnt[N] = 0;
+      continue;
+    }
+    int c = static_cast<int>(m * chunks / N);  // chunk c starts at term N c / chunks (rounded down)
+    while (c + 1 < chunks && N * (c + 1) / chunks <= m) ++c;
+    while (N * c / chunks > m) --c;
+    const bool start = m == N * c / chunks, end = m + 1 == N * (c + 1) / chunks;
+    const uint16_t* a = support + m * D;
+    const uint16_t* b = a - D;  // the previous term (not read at a chunk's start)
+    int common = 0;             // axes that agree with the previous term
+    if (!start)
+      while (common < D && a[common] == b[common]) ++common;
+    int opens = 0, own = 0, closes = 0;
+    for (int i = 0; i < D; ++i) {
+      const bool nz = a[i] != 0;
+      own += nz;
+      opens += nz && i >= common;
+      closes += !start && i >= common && b[i] != 0;
+    }
+    if (!fill) {
+      cnt[m] = closes + 1 + (end ? own : 0);
+      most = max(most, own);
+      continue;
+    }
+    uint32_t* w = prog + cnt[m];
+    if (start) word[c] = cnt[m];
+    if (!start)
+      for (int i = D - 1; i >= common; --i)
+        if (b[i] != 0) *w++ = 0x80000000u | static_cast<uint32_t>(i * tk + b[i]);
+    *w++ = static_cast<uint32_t>(opens);
+    if (end)
+      for (int i = D - 1; i >= 0; --i)
+        if (a[i] != 0) *w++ = 0x80000000u | static_cast<uint32_t>(i * tk + a[i]);
+  }
+  if (fill) return;
+  atomicMax(&s_most, most);
+  __syncthreads();
+  if (threadIdx.x == 0) atomicMax(word + chunks + 1, s_most);
+}
+
 fct_status cuda_err(cudaError_t e, const char* what) {
   if (e == cudaErrorMemoryAllocation) return fail(FCT_ERR_OOM, std::string(what) + ": " + cudaGetErrorString(e));
   return fail(FCT_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
@@ -679,6 +734,20 @@ void radix_sort(int32_t** k, int32_t** v, int32_t** k2, int32_t** v2, int64_t n,
 }
 
 }  // namespace
+
+fct_status build_eval_program(const uint16_t* d_support, int64_t N, int D, int tk, int chunks, uint32_t* prog,
+                              int32_t* word, void* scratch, void* stream) {
+  const cudaStream_t st = static_cast<cudaStream_t>(stream);
+  const int64_t nparts = (N + 1 + kScanTile - 1) / kScanTile + 1;
+  int32_t* cnt = static_cast<int32_t*>(scratch);  // counts, scan partials, total: N + N / 2048 + 5 words at most
+  int32_t *part = cnt + N + 1, *total = part + nparts;
+  cudaMemsetAsync(word + chunks + 1, 0, sizeof(int32_t), st);
+  eval_words_kernel<<<elem_blocks(N + 1), kElemThreads, 0, st>>>(N, D, tk, chunks, d_support, false, cnt, prog, word);
+  exclusive_scan(cnt, cnt, N + 1, part, total, st);
+  eval_words_kernel<<<elem_blocks(N + 1), kElemThreads, 0, st>>>(N, D, tk, chunks, d_support, true, cnt, prog, word);
+  const cudaError_t e = cudaGetLastError();
+  return e == cudaSuccess ? FCT_OK : cuda_err(e, "evaluation program");
+}
 
 void DeviceTables::release() {
   if (mem) {
