@@ -376,9 +376,8 @@ __device__ __noinline__ float2 cells_task(const DevPlan& P, unsigned char* dsm, 
 // s = right-hand side, x = 0, gamma0 = |s|^2; returns as cg_normal does.  s and p
 // are the halves of sp32, tpart lives in y0 and the per-task and per-chunk
 // partials in y1 (the DCT's buffers, free by now).
-// Not inlined: the calls inside would cost the solver's other paths registers.
 template <int BT>
-__device__ __noinline__ bool cg_cells(const DevPlan& P, Team& team, unsigned char* dsm, double gamma0, double tol, int max_iter,
+__device__ bool cg_cells(const DevPlan& P, Team& tm, unsigned char* dsm, double gamma0, double tol, int max_iter,
                          int stall, int* iters_out, double* gamma_out, int* status_out) {
   constexpr int NW = BT / 32;
   __shared__ float2 wpart[kUnitGroup][NW];
@@ -393,7 +392,6 @@ __device__ __noinline__ bool cg_cells(const DevPlan& P, Team& team, unsigned cha
     return true;
   }
   const int N = P.N, K = P.K, NG = P.tk_groups, GG = P.tk_gg;
-  Team tm = team;  // its fields in registers
   const int64_t NP = P.tk_np;
   const int CW = P.tk_cw, LG = P.tk_lg, nown = P.tk_nown;
   const int tid = static_cast<int>(threadIdx.x), warp = tid >> 5, lane = tid & 31;
@@ -551,7 +549,6 @@ __device__ __noinline__ bool cg_cells(const DevPlan& P, Team& team, unsigned cha
     }
     first = false;
   }
-  team.epoch = tm.epoch;
   if (tid == 0) {
     sh_ctl[1] = ctl >= 16 ? ctl - 16 : FCT_OK;
     sh_ctl[2] = it;

@@ -34,7 +34,7 @@ __device__ __forceinline__ int ld_volatile_i32(const int* p) {
 }
 
 // Loads of data written earlier in the same launch by other blocks bypass L1
-// (ldcg), except the CG gathers of {s, p} and q: those vectors change only in
+// (ldcg), except the CG gathers of s and q: those vectors change only in
 // the phase before a team barrier, and the barrier's gpu-scope acquire drops
 // the SM's L1 lines, so plain loads are current and repeated sectors hit L1.
 template <typename T>
@@ -363,10 +363,6 @@ __device__ __forceinline__ V lane_group_sum(V v, int L) {
   return v;
 }
 
-
-template <typename V> struct Vec2;
-template <> struct Vec2<double> { using T = double2; };
-template <> struct Vec2<float> { using T = float2; };
 
 struct SolveArgs {
   SolveJob single;          // used when jobs == nullptr

@@ -193,12 +193,12 @@ struct DevPlan {
   double* b;                 // [R]
   double* rres;              // [R] FP64 residual b - A x (mixed path sweeps)
   double* q;                 // [R]
-  double2* sp;               // [N] {s, p} interleaved: one 16-byte gather per entry
+  double2* sp;               // [N] s, then p (N doubles each)
   double* part_r;            // [n_row_units]    FP64 per-unit partial sums (|q|^2 and the set-up phases)
   double* part_c;            // [n_coef_chunks]  (|s|^2 and the refinement sweeps)
   // FP32 workspace of the mixed path
   float* q32;                // [R]
-  float2* sp32;              // [N] {s, p} of the inner FP32 solve
+  float2* sp32;              // [N] s, then p of the inner FP32 solve
   float* dx32;               // [N]
   // normal matrix W = A^T A of the mixed path's inner solve (n_w_units = 0:
   // not built; the inner solve then applies A and A^T in two phases)

@@ -386,19 +386,22 @@ __device__ __forceinline__ V row_gather(const DevPlan& P, const BlockTabs& T, co
   return a;
 }
 
-// Phase-A gather of the interleaved {s, p}: as = sum w s[col], ap = sum w p[col]
-// (ap skipped on the first iteration, when p is not defined yet).
-template <typename V, typename V2, typename WT, bool SV, int EPR>
-__device__ __forceinline__ void row_gather_sp(const DevPlan& P, const BlockTabs& T, const WT* __restrict__ w, int u,
-                                             int k, int wk, int* row_out, bool* lead, const V2* sp, bool first, V* as,
-                                             V* ap) {
+// Phase-A gather: as = sum w s[col], and the row's previous q (skipped on the
+// first iteration, when there is none), loaded by the lead lane beside the
+// gather's first loads.
+template <typename V, typename WT, bool SV, int EPR>
+__device__ __forceinline__ void row_gather_s(const DevPlan& P, const BlockTabs& T, const WT* __restrict__ w, int u,
+                                            int k, int wk, int* row_out, bool* lead, const V* s, const V* q, bool first,
+                                            V* as, V* q_old) {
   const RowUnit g = row_unit_geom<SV>(P, T, u, k);
   const bool ws = SV && g.wt != nullptr && static_cast<int>(sizeof(WT)) == T.wbytes;
   const bool wide = g.lc > 32;  // see row_gather_n
   const int gl = wide ? P.workers : g.lc;
   const int row = wide ? g.r0 : g.r0 + wk / g.lc;
   const int lane = wide ? wk : (wk & (g.lc - 1));
-  V a1 = V(0), a2 = V(0);
+  const bool is_lead = (row < g.r1) && (lane & (wide ? 31 : g.lc - 1)) == 0;
+  V a1 = V(0);
+  *q_old = !first && is_lead ? ldcg(q + row) : V(0);
   if (row < g.r1) {
     int ja, jb;
     if (g.rp) {
@@ -420,15 +423,12 @@ __device__ __forceinline__ void row_gather_sp(const DevPlan& P, const BlockTabs&
           c[i] = cl[j];
           wv[i] = ws ? wp[j] : __ldg(wp + j);
         }
-        V2 v[EPR];
+        V v[EPR];
 #pragma unroll
-        for (int i = 0; i < EPR; ++i) v[i] = sp[c[i]];
+        for (int i = 0; i < EPR; ++i) v[i] = s[c[i]];
 #pragma unroll
         for (int i = 0; i < EPR; ++i)
-          if (j0 + i * gl < jb) {
-            a1 = fma(static_cast<V>(wv[i]), v[i].x, a1);
-            if (!first) a2 = fma(static_cast<V>(wv[i]), v[i].y, a2);
-          }
+          if (j0 + i * gl < jb) a1 = fma(static_cast<V>(wv[i]), v[i], a1);
       }
     } else {
       for (int j0 = ja + lane; j0 < jb; j0 += EPR * gl) {
@@ -440,22 +440,18 @@ __device__ __forceinline__ void row_gather_sp(const DevPlan& P, const BlockTabs&
           c[i] = __ldg(P.col + j);
           wv[i] = __ldg(w + j);
         }
-        V2 v[EPR];
+        V v[EPR];
 #pragma unroll
-        for (int i = 0; i < EPR; ++i) v[i] = sp[c[i]];
+        for (int i = 0; i < EPR; ++i) v[i] = s[c[i]];
 #pragma unroll
         for (int i = 0; i < EPR; ++i)
-          if (j0 + i * gl < jb) {
-            a1 = fma(static_cast<V>(wv[i]), v[i].x, a1);
-            if (!first) a2 = fma(static_cast<V>(wv[i]), v[i].y, a2);
-          }
+          if (j0 + i * gl < jb) a1 = fma(static_cast<V>(wv[i]), v[i], a1);
       }
     }
   }
   *as = lane_group_sum(a1, wide ? 32 : g.lc);
-  *ap = lane_group_sum(a2, wide ? 32 : g.lc);
   *row_out = row;
-  *lead = (row < g.r1) && (lane & (wide ? 31 : g.lc - 1)) == 0;
+  *lead = is_lead;
 }
 
 // Wide rows sort first and are one unit each, so they are the first
@@ -595,10 +591,11 @@ __device__ __forceinline__ bool coef_owner(const DevPlan& P, int c, int wk, int*
 //   q = A p;  alpha = |s|^2/|q|^2;  x += alpha p;  s -= alpha A^T q;
 //   beta = |s|^2_new / |s|^2;  p = s + beta p.
 // One team barrier per matrix product:
-//   phase A: q = A s + beta A p from one 16-byte gather of {s, p} per entry,
-//            while warp 0 reduces |s|^2 of the previous phase B;
+//   phase A: q = A s + beta q_old (= A p), so only s is gathered: half the bytes
+//            and, for FP64, half the multiply-adds of a gather of {s, p};
+//            meanwhile warp 0 reduces |s|^2 of the previous phase B;
 //   phase B: t = A^T q while warp 0 reduces |q|^2; the coefficient owner
-//            then writes {s - alpha t, s + beta p} and x + alpha p in place.
+//            then writes s - alpha t, p = s + beta p and x + alpha p in place.
 // Workers stream through the block's units without block-wide syncs; each
 // unit's partial is the fixed-order sum of its warps' sums, so partials (and
 // the result) do not depend on the team size.
@@ -611,7 +608,7 @@ __device__ __forceinline__ bool coef_owner(const DevPlan& P, int c, int wk, int*
 // near 1/sqrt(gamma0) (exact), which keeps the FP32 squares of late
 // iterations in range.  alpha, beta and the stopping test are computed once
 // per block by one thread and broadcast.
-// On entry sp[m].x = right-hand side, x = 0, gamma0 = |s|^2 (> 0).  Stops when
+// On entry s = right-hand side, x = 0, gamma0 = |s|^2 (> 0).  Stops when
 // gamma <= tol^2 gamma0, after max_iter (FCT_ERR_NOCONV) or, if stall > 0,
 // when gamma has not decreased for `stall` iterations.  All threads of all
 // blocks return the same iteration count, final gamma and status.
@@ -636,9 +633,8 @@ template <> __device__ __forceinline__ float2 sc_of<float2>(double v) { return d
 
 template <int BT, typename V, typename WT, typename XT, bool SV, int DEEP>
 __device__ bool cg_normal(const DevPlan& P, Team& tm, const BlockTabs& T, const WT* wcsr, const WT* wcm,
-                          typename Vec2<V>::T* sp, V* q, XT* x, double gamma0, double tol, int max_iter, int stall,
+                          V* s, V* p, V* q, XT* x, double gamma0, double tol, int max_iter, int stall,
                           int* iters_out, double* gamma_out, int* status_out, double* red) {
-  using V2 = typename Vec2<V>::T;
   using PT = typename SqPart<V>::T;
   constexpr int NW = BT / 32 - 1;  // worker warps
   __shared__ PT wpart[kUnitGroup][NW];
@@ -666,6 +662,9 @@ __device__ bool cg_normal(const DevPlan& P, Team& tm, const BlockTabs& T, const 
   V best = sc_val(gam);
   int it = 0, best_it = 0;
   bool first = true;
+  // the condition probe forms A p from p itself: its start vector may have a part
+  // that A maps to zero, where q's recurrence would divide by a vanishing |q|^2
+  const bool probe = sizeof(V) == 8 && P.s_init != nullptr;
   // lead lanes of a unit sit at multiples of its lanes per row (coefficient)
   auto warp_part = [&](int kk, PT v, int lc) {
     v = warp_sum_from(v, lc);
@@ -690,15 +689,15 @@ __device__ bool cg_normal(const DevPlan& P, Team& tm, const BlockTabs& T, const 
   for (int pass = 0;; ++pass) {
     // ================= phase A: q = A s + beta A p
     {
-      auto gather_a = [&](int u, int k, V* as, V* ap, int* row, bool* lead) {
-        row_gather_sp<V, V2, WT, SV, (4 << DEEP)>(P, T, wcsr, u, k, wk, row, lead, sp, first, as, ap);
+      auto gather_a = [&](int u, int k, V* as, V* qo, int* row, bool* lead) {
+        row_gather_s<V, WT, SV, (4 << DEEP)>(P, T, wcsr, u, k, wk, row, lead, s, q, first, as, qo);
       };
       int u = tm.rank;
-      V as = V(0), ap = V(0);
+      V as = V(0), qo = V(0);
       int row = 0;
       bool lead = false;
       if (wk >= 0) {
-        if (u < nru) gather_a(u, 0, &as, &ap, &row, &lead);
+        if (u < nru && !probe) gather_a(u, 0, &as, &qo, &row, &lead);
       } else {
         PT gnew = gam;
         if (!first) gnew = warp0_sum(part_c, ncc);
@@ -734,11 +733,18 @@ __device__ bool cg_normal(const DevPlan& P, Team& tm, const BlockTabs& T, const 
       const V beta = sh_ab[0];
       int k = 0, kg = 0, u0 = u;
       for (; u < nru; u += tm.G, ++k) {
-        if (k > 0 && wk >= 0) gather_a(u, k, &as, &ap, &row, &lead);
-        if (u < nwide) wide_row_combine<NW>(wk, &as, &ap, &lead);
+        if (probe && wk >= 0) {
+          if constexpr (sizeof(V) == 8)
+            as = row_gather<V, WT, SV, (4 << DEEP)>(P, T, wcsr, u, k, wk, &row, &lead,
+                                                    [&](int i) { return first ? s[i] : fma(beta, p[i], s[i]); });
+        } else if (k > 0 && wk >= 0) {
+          gather_a(u, k, &as, &qo, &row, &lead);
+        }
+        V unused = V(0);
+        if (u < nwide) wide_row_combine<NW>(wk, &as, &unused, &lead);
         PT part = pzero_part(PT{});
         if (wk >= 0 && lead) {
-          const V qv = first ? as : fma(beta, ap, as);
+          const V qv = first || probe ? as : fma(beta, qo, as);
           stcg(q + row, qv);
           part = sq_part(qv, rs);
         }
@@ -751,13 +757,14 @@ __device__ bool cg_normal(const DevPlan& P, Team& tm, const BlockTabs& T, const 
       }
       if (!phase_end<NW>(tm, wpart, part_r, u0, kg)) return false;
     }
-    // ================= phase B: t = A^T q; {s, p} and x updated by the owner
+    // ================= phase B: t = A^T q; s, p and x updated by the owner
     {
       const int L = P.coef_split ? 1 : P.coef_lanes;  // lead lanes sit at multiples of L
-      auto own_load = [&](int c, V2* o, XT* xo) {
+      auto own_load = [&](int c, V* so, V* po, XT* xo) {
         int m = 0;
         if (coef_owner(P, c, wk, &m) && m < P.N) {
-          *o = ldcg(sp + m);
+          *so = ldcg(s + m);
+          if (!first) *po = ldcg(p + m);
           *xo = ldcg(x + m);
         }
       };
@@ -765,11 +772,11 @@ __device__ bool cg_normal(const DevPlan& P, Team& tm, const BlockTabs& T, const 
       V t = V(0);
       int m = 0;
       bool lead = false;
-      V2 o{};
+      V so = V(0), po = V(0);
       XT xo = XT(0);
       if (wk >= 0) {
         if (c < ncc) {
-          own_load(c, &o, &xo);
+          own_load(c, &so, &po, &xo);
           t = coef_gather<V, WT, SV, (8 << DEEP)>(P, T, wcm, c, 0, wk, &m, &lead, [&](int i) { return q[i]; });
         }
       } else {
@@ -793,18 +800,16 @@ __device__ bool cg_normal(const DevPlan& P, Team& tm, const BlockTabs& T, const 
       int k = 0, kg = 0, c0 = c;
       for (; c < ncc; c += tm.G, ++k) {
         if (k > 0 && wk >= 0) {
-          own_load(c, &o, &xo);
+          own_load(c, &so, &po, &xo);
           t = coef_gather<V, WT, SV, (8 << DEEP)>(P, T, wcm, c, k, wk, &m, &lead, [&](int i) { return q[i]; });
         }
         t = coef_combine<NW>(P, T, t, k, wk, m, &lead);
         PT part = pzero_part(PT{});
         if (wk >= 0 && lead) {
-          const V pn = first ? o.x : fma(beta, o.y, o.x);
-          const V sn = fma(-alpha, t, o.x);
-          V2 nv;
-          nv.x = sn;
-          nv.y = pn;
-          stcg(sp + m, nv);
+          const V pn = first ? so : fma(beta, po, so);
+          const V sn = fma(-alpha, t, so);
+          stcg(s + m, sn);
+          stcg(p + m, pn);
           stcg(x + m, static_cast<XT>(fma(static_cast<XT>(alpha), static_cast<XT>(pn), xo)));
           part = sq_part(sn, rs);
         }
@@ -841,7 +846,7 @@ __device__ bool cg_normal(const DevPlan& P, Team& tm, const BlockTabs& T, const 
 // form needs a barrier after A p and another after A^T q).
 //   vectors (FP32, owned by the thread group of their row): r, p, s = W p,
 //   z = W s, w = W r (two buffers: one is gathered while the next is written),
-//   x = dx32; right-hand side: sp32[m].x; start x = 0.
+//   x = dx32; right-hand side: s, the first half of sp32; start x = 0.
 //   per iteration, with gamma = r.r, delta = w.r from the previous barrier:
 //     beta = gamma / gamma_prev, alpha = gamma / (delta - beta gamma / alpha_prev)
 //     z = y + beta z, s = w + beta s, p = r + beta p
@@ -877,7 +882,7 @@ __device__ bool pcg_normal_w(const DevPlan& P, Team& tm, const BlockTabs& T, dou
   float* const vs = P.wv + 4 * static_cast<size_t>(N);
   float* const vz = P.wv + 5 * static_cast<size_t>(N);
   float* const vx = P.dx32;
-  const float* const rhs = reinterpret_cast<const float*>(P.sp32);  // .x of {s, p}: stride 2
+  const float* const rhs = reinterpret_cast<const float*>(P.sp32);  // s, the first half
   // thread 0's state
   double gam_prev = 1.0, al_prev = 1.0, best = 1.0e300, gam_last = 1.0;
   int best_it = 0;
@@ -940,10 +945,10 @@ __device__ bool pcg_normal_w(const DevPlan& P, Team& tm, const BlockTabs& T, dou
       int m = 0;
       bool lead = false;
       float y = 0.0f;
-      if (wk >= 0) y = gather(u, k, rhs, 2, &m, &lead);
+      if (wk >= 0) y = gather(u, k, rhs, 1, &m, &lead);
       double2 part = make_double2(0.0, 0.0);
       if (wk >= 0 && lead) {
-        const float r = ldcg(rhs + 2 * static_cast<size_t>(m));
+        const float r = ldcg(rhs + m);
         stcg(vr + m, r);
         stcg(wb0 + m, y);
         stcg(vx + m, 0.0f);
@@ -1112,6 +1117,9 @@ __device__ bool solve_job(const SolveJob& J, Team& tm, double* red, unsigned cha
   }
   load_block_tabs<BT>(P, tm, dsm, smem_bytes, &T, J.precision == FCT_MIXED && P.n_w_units > 0 && P.s_init == nullptr,
                       SV ? (J.precision == FCT_MIXED ? 4 : 8) : 0, !cells);
+  // s and p of the CG solves are the halves of sp and sp32
+  double* const s64 = reinterpret_cast<double*>(P.sp);
+  float* const s32 = reinterpret_cast<float*>(P.sp32);
   const int ncc = P.n_coef_chunks, nre = P.n_rowel_chunks, nru = P.n_row_units, nwide = P.n_wide_units;
   const int wk = static_cast<int>(threadIdx.x) - 32;
   const int nce = (P.N + BT - 1) / BT;  // elementwise units over coefficients
@@ -1122,7 +1130,7 @@ __device__ bool solve_job(const SolveJob& J, Team& tm, double* red, unsigned cha
       double part = 0.0;
       if (m < P.N) {
         const double v = __ldg(P.s_init + m);
-        stcg(P.sp + m, make_double2(v, 0.0));
+        stcg(s64 + m, v);
         stcg(J.coeffs + m, 0.0);
         part = v * v;
       }
@@ -1162,7 +1170,7 @@ __device__ bool solve_job(const SolveJob& J, Team& tm, double* red, unsigned cha
       t = coef_combine<BT / 32 - 1>(P, T, t, k, wk, m, &lead);
       double part = 0.0;
       if (lead) {
-        stcg(P.sp + m, make_double2(t, 0.0));
+        stcg(s64 + m, t);
         part = t * t;
       }
       part = block_sum<BT>(part, red);
@@ -1178,7 +1186,7 @@ __device__ bool solve_job(const SolveJob& J, Team& tm, double* red, unsigned cha
   if (!isfinite(gamma0)) {
     status = FCT_ERR_NONFINITE;
   } else if (J.precision != FCT_MIXED) {
-    if (!cg_normal<BT, double, double, double, SV, DEEP>(P, tm, T, P.wcsr, P.wcm, P.sp, P.q, J.coeffs, gamma0, J.tol,
+    if (!cg_normal<BT, double, double, double, SV, DEEP>(P, tm, T, P.wcsr, P.wcm, s64, s64 + P.N, P.q, J.coeffs, gamma0, J.tol,
                                                J.max_iter, 0, &iters, &gfinal, &status, red))
       return false;
   } else if (gamma0 > 0.0) {
@@ -1190,9 +1198,7 @@ __device__ bool solve_job(const SolveJob& J, Team& tm, double* red, unsigned cha
     for (int u = tm.rank; u < nce; u += tm.G) {
       const int m = u * BT + threadIdx.x;
       if (m < P.N) {
-        const float v = static_cast<float>(ldcg(P.sp + m).x * ci);
-        if (cells) stcg(reinterpret_cast<float*>(P.sp32) + m, v);  // cg_cells keeps s contiguous
-        else stcg(P.sp32 + m, make_float2(v, 0.0f));
+        stcg(s32 + m, static_cast<float>(ldcg(s64 + m) * ci));
         stcg(P.dx32 + m, 0.0f);
       }
     }
@@ -1210,7 +1216,7 @@ __device__ bool solve_job(const SolveJob& J, Team& tm, double* red, unsigned cha
           if (!cg_cells<BT>(P, tm, dsm, g64 * ci * ci, J.inner_tol, J.max_iter, 64, &it_in, &g_in, &st_in))
             return false;
         }
-      } else if (!cg_normal<BT, float, float, float, SV, DEEP>(P, tm, T, P.wcsr32, P.wcm32, P.sp32, P.q32, P.dx32,
+      } else if (!cg_normal<BT, float, float, float, SV, DEEP>(P, tm, T, P.wcsr32, P.wcm32, s32, s32 + P.N, P.q32, P.dx32,
                                                      g64 * ci * ci, J.inner_tol, J.max_iter, 64, &it_in, &g_in,
                                                      &st_in, red)) {
         return false;
@@ -1248,9 +1254,8 @@ __device__ bool solve_job(const SolveJob& J, Team& tm, double* red, unsigned cha
         t = coef_combine<BT / 32 - 1>(P, T, t, kc, wk, m, &lead);
         double part = 0.0;
         if (lead) {
-          if (cells) stcg(reinterpret_cast<float*>(P.sp32) + m, static_cast<float>(t * ci));
-          else stcg(P.sp32 + m, make_float2(static_cast<float>(t * ci), 0.0f));
-          stcg(P.sp + m, make_double2(t, 0.0));  // for an FP64 continuation
+          stcg(s32 + m, static_cast<float>(t * ci));
+          stcg(s64 + m, t);  // for an FP64 continuation
           stcg(P.dx32 + m, 0.0f);
           part = t * t;
         }
@@ -1273,7 +1278,7 @@ __device__ bool solve_job(const SolveJob& J, Team& tm, double* red, unsigned cha
         int it64 = 0, st64 = FCT_OK;
         double g_out = g64;
         const double tol_eff = J.tol * sqrt(gamma0 / g64);
-        if (!cg_normal<BT, double, double, double, SV, DEEP>(P, tm, T, P.wcsr, P.wcm, P.sp, P.q, x, g64, tol_eff, J.max_iter,
+        if (!cg_normal<BT, double, double, double, SV, DEEP>(P, tm, T, P.wcsr, P.wcm, s64, s64 + P.N, P.q, x, g64, tol_eff, J.max_iter,
                                                    0, &it64, &g_out, &st64, red))
           return false;
         iters += it64;
