@@ -118,9 +118,7 @@ static __device__ void team_exit(const Team& tm) {
 // and its lane 0 arrives at and waits on the team barrier, so one block-wide
 // sync before and one after cover both the flush and the barrier.
 __device__ __forceinline__ double padd(double a, double b) { return a + b; }
-__device__ __forceinline__ double2 padd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ double pzero(double) { return 0.0; }
-__device__ __forceinline__ double2 pzero(double2) { return make_double2(0.0, 0.0); }
 
 // ---------------------------------------------------------------------------
 // Sums of squares of FP32 vectors at FP64 accuracy on the FP32 pipe
@@ -185,7 +183,6 @@ __device__ __forceinline__ float2 warp_sum_from(float2 v, int lc) {
   return v;
 }
 __device__ __forceinline__ double widen(double v) { return v; }
-__device__ __forceinline__ double2 widen(double2 v) { return v; }
 __device__ __forceinline__ double widen(float2 v) { return static_cast<double>(v.x) + static_cast<double>(v.y); }
 
 // Per-warp partial of a sum of squares: FP64 for FP64 vectors, a double-float
@@ -203,6 +200,20 @@ __device__ __forceinline__ float2 pzero_part(float2) { return make_float2(0.0f, 
 
 __device__ __forceinline__ float2 padd(float2 a, float2 b) { return df_add(a, b); }
 __device__ __forceinline__ float2 pzero(float2) { return make_float2(0.0f, 0.0f); }
+
+// Two double-float pairs side by side (the pipelined CG's two inner products).
+__device__ __forceinline__ float4 padd(float4 a, float4 b) {
+  const float2 u = df_add(make_float2(a.x, a.y), make_float2(b.x, b.y));
+  const float2 v = df_add(make_float2(a.z, a.w), make_float2(b.z, b.w));
+  return make_float4(u.x, u.y, v.x, v.y);
+}
+__device__ __forceinline__ float4 warp_sum(float4 v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+    v = padd(v, make_float4(__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o),
+                            __shfl_xor_sync(0xffffffffu, v.z, o), __shfl_xor_sync(0xffffffffu, v.w, o)));
+  return v;
+}
 
 // Sum of a unit's NW per-warp partials: a tree over values loaded side by side
 // (a chain of NW dependent additions is on the path to every team barrier).
@@ -320,24 +331,19 @@ __device__ __forceinline__ float2 warp0_sum(const float2* part, int n) {
   return warp_sum(s);
 }
 
-// Warp 0: FP64 pair sums of n partials in a fixed order (lane 0 holds the result).
-__device__ __forceinline__ double2 warp0_sum(const double2* part, int n) {
-  double2 v = make_double2(0.0, 0.0);
-  for (int i0 = threadIdx.x; i0 < n; i0 += 32 * 4) {
-    double2 t[4];
+// Warp 0: sums of n partials of two double-float pairs in a fixed order (every lane).
+__device__ __forceinline__ float4 warp0_sum(const float4* part, int n) {
+  const float4 zero = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  float4 v = zero;
+  for (int i0 = threadIdx.x; i0 < n; i0 += 32 * 8) {
+    float4 t[8];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) t[j] = ldcg(part + min(i0 + 32 * j, n - 1));  // every load issued
+    for (int j = 0; j < 8; ++j) t[j] = ldcg(part + min(i0 + 32 * j, n - 1));  // every load issued
 #pragma unroll
-    for (int j = 0; j < 4; ++j) t[j] = i0 + 32 * j < n ? t[j] : make_double2(0.0, 0.0);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) v = padd(v, t[j]);
+    for (int j = 0; j < 8; ++j) t[j] = i0 + 32 * j < n ? t[j] : zero;
+    v = padd(v, padd(padd(padd(t[0], t[1]), padd(t[2], t[3])), padd(padd(t[4], t[5]), padd(t[6], t[7]))));
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
-    v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
-  }
-  return v;
+  return warp_sum(v);
 }
 
 // All threads: team sum of n partials (used outside the overlapped phases).

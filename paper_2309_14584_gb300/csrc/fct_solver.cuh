@@ -386,7 +386,79 @@ __device__ __forceinline__ V row_gather(const DevPlan& P, const BlockTabs& T, co
   return a;
 }
 
-// Phase-A gather: as = sum w s[col], and the row's previous q (skipped on the
+// Phase-A gather of the FP32 solves, interleaved {s, p}: as = sum w s[col], ap = sum w p[col]
+// (ap skipped on the first iteration, when p is not defined yet).
+template <typename V, typename V2, typename WT, bool SV, int EPR>
+__device__ __forceinline__ void row_gather_sp(const DevPlan& P, const BlockTabs& T, const WT* __restrict__ w, int u,
+                                             int k, int wk, int* row_out, bool* lead, const V2* sp, bool first, V* as,
+                                             V* ap) {
+  const RowUnit g = row_unit_geom<SV>(P, T, u, k);
+  const bool ws = SV && g.wt != nullptr && static_cast<int>(sizeof(WT)) == T.wbytes;
+  const bool wide = g.lc > 32;  // see row_gather_n
+  const int gl = wide ? P.workers : g.lc;
+  const int row = wide ? g.r0 : g.r0 + wk / g.lc;
+  const int lane = wide ? wk : (wk & (g.lc - 1));
+  V a1 = V(0), a2 = V(0);
+  if (row < g.r1) {
+    int ja, jb;
+    if (g.rp) {
+      ja = g.rp[row - g.r0];
+      jb = g.rp[row - g.r0 + 1];
+    } else {
+      ja = __ldg(P.rowptr + row);
+      jb = __ldg(P.rowptr + row + 1);
+    }
+    if (g.cl) {
+      const int* cl = g.cl;
+      const WT* wp = ws ? static_cast<const WT*>(g.wt) : w + g.jbase;
+      for (int j0 = ja + lane; j0 < jb; j0 += EPR * gl) {
+        int c[EPR];
+        WT wv[EPR];
+#pragma unroll
+        for (int i = 0; i < EPR; ++i) {
+          const int j = min(j0 + i * gl, jb - 1);
+          c[i] = cl[j];
+          wv[i] = ws ? wp[j] : __ldg(wp + j);
+        }
+        V2 v[EPR];
+#pragma unroll
+        for (int i = 0; i < EPR; ++i) v[i] = sp[c[i]];
+#pragma unroll
+        for (int i = 0; i < EPR; ++i)
+          if (j0 + i * gl < jb) {
+            a1 = fma(static_cast<V>(wv[i]), v[i].x, a1);
+            if (!first) a2 = fma(static_cast<V>(wv[i]), v[i].y, a2);
+          }
+      }
+    } else {
+      for (int j0 = ja + lane; j0 < jb; j0 += EPR * gl) {
+        int c[EPR];
+        WT wv[EPR];
+#pragma unroll
+        for (int i = 0; i < EPR; ++i) {
+          const int j = min(j0 + i * gl, jb - 1);
+          c[i] = __ldg(P.col + j);
+          wv[i] = __ldg(w + j);
+        }
+        V2 v[EPR];
+#pragma unroll
+        for (int i = 0; i < EPR; ++i) v[i] = sp[c[i]];
+#pragma unroll
+        for (int i = 0; i < EPR; ++i)
+          if (j0 + i * gl < jb) {
+            a1 = fma(static_cast<V>(wv[i]), v[i].x, a1);
+            if (!first) a2 = fma(static_cast<V>(wv[i]), v[i].y, a2);
+          }
+      }
+    }
+  }
+  *as = lane_group_sum(a1, wide ? 32 : g.lc);
+  *ap = lane_group_sum(a2, wide ? 32 : g.lc);
+  *row_out = row;
+  *lead = (row < g.r1) && (lane & (wide ? 31 : g.lc - 1)) == 0;
+}
+
+// Phase-A gather of the FP64 solves: as = sum w s[col], and the row's previous q (skipped on the
 // first iteration, when there is none), loaded by the lead lane beside the
 // gather's first loads.
 template <typename V, typename WT, bool SV, int EPR>
@@ -591,9 +663,13 @@ __device__ __forceinline__ bool coef_owner(const DevPlan& P, int c, int wk, int*
 //   q = A p;  alpha = |s|^2/|q|^2;  x += alpha p;  s -= alpha A^T q;
 //   beta = |s|^2_new / |s|^2;  p = s + beta p.
 // One team barrier per matrix product:
-//   phase A: q = A s + beta q_old (= A p), so only s is gathered: half the bytes
-//            and, for FP64, half the multiply-adds of a gather of {s, p};
-//            meanwhile warp 0 reduces |s|^2 of the previous phase B;
+//   phase A: FP64: q = A s + beta q_old (= A p), so only s is gathered: half the
+//            bytes and half the multiply-adds of a gather of {s, p} (D = 10
+//            degree 8: 14.7 -> 13.1 ms).  FP32: q = A s + beta A p from one 8-byte
+//            gather of {s, p} per entry: by the recurrence some ill-conditioned
+//            inner solves left the residual so far off that a fourth sweep was
+//            needed (first-kind D = 6: 1776 iterations against 1232).  Meanwhile
+//            warp 0 reduces |s|^2 of the previous phase B;
 //   phase B: t = A^T q while warp 0 reduces |q|^2; the coefficient owner
 //            then writes s - alpha t, p = s + beta p and x + alpha p in place.
 // Workers stream through the block's units without block-wide syncs; each
@@ -608,7 +684,7 @@ __device__ __forceinline__ bool coef_owner(const DevPlan& P, int c, int wk, int*
 // near 1/sqrt(gamma0) (exact), which keeps the FP32 squares of late
 // iterations in range.  alpha, beta and the stopping test are computed once
 // per block by one thread and broadcast.
-// On entry s = right-hand side, x = 0, gamma0 = |s|^2 (> 0).  Stops when
+// On entry s (FP32: sp[m].x) = right-hand side, x = 0, gamma0 = |s|^2 (> 0).  Stops when
 // gamma <= tol^2 gamma0, after max_iter (FCT_ERR_NOCONV) or, if stall > 0,
 // when gamma has not decreased for `stall` iterations.  All threads of all
 // blocks return the same iteration count, final gamma and status.
@@ -633,10 +709,14 @@ template <> __device__ __forceinline__ float2 sc_of<float2>(double v) { return d
 
 template <int BT, typename V, typename WT, typename XT, bool SV, int DEEP>
 __device__ bool cg_normal(const DevPlan& P, Team& tm, const BlockTabs& T, const WT* wcsr, const WT* wcm,
-                          V* s, V* p, V* q, XT* x, double gamma0, double tol, int max_iter, int stall,
+                          V* s, V* q, XT* x, double gamma0, double tol, int max_iter, int stall,
                           int* iters_out, double* gamma_out, int* status_out, double* red) {
   using PT = typename SqPart<V>::T;
+  using V2 = float2;
   constexpr int NW = BT / 32 - 1;  // worker warps
+  constexpr bool kRec = sizeof(V) == 8;  // q by its recurrence; FP32: {s, p} interleaved at s
+  V* const p = s + P.N;                  // FP64: s, then p
+  V2* const sp = reinterpret_cast<V2*>(s);
   __shared__ PT wpart[kUnitGroup][NW];
   __shared__ V sh_ab[2];           // beta, alpha
   __shared__ double sh_gam;
@@ -690,7 +770,10 @@ __device__ bool cg_normal(const DevPlan& P, Team& tm, const BlockTabs& T, const 
     // ================= phase A: q = A s + beta A p
     {
       auto gather_a = [&](int u, int k, V* as, V* qo, int* row, bool* lead) {
-        row_gather_s<V, WT, SV, (4 << DEEP)>(P, T, wcsr, u, k, wk, row, lead, s, q, first, as, qo);
+        if constexpr (kRec)
+          row_gather_s<V, WT, SV, (4 << DEEP)>(P, T, wcsr, u, k, wk, row, lead, s, q, first, as, qo);
+        else
+          row_gather_sp<V, V2, WT, SV, (4 << DEEP)>(P, T, wcsr, u, k, wk, row, lead, sp, first, as, qo);
       };
       int u = tm.rank;
       V as = V(0), qo = V(0);
@@ -740,8 +823,9 @@ __device__ bool cg_normal(const DevPlan& P, Team& tm, const BlockTabs& T, const 
         } else if (k > 0 && wk >= 0) {
           gather_a(u, k, &as, &qo, &row, &lead);
         }
+        // qo: FP64 the row's previous q; FP32 the gather of p, summed like that of s
         V unused = V(0);
-        if (u < nwide) wide_row_combine<NW>(wk, &as, &unused, &lead);
+        if (u < nwide) wide_row_combine<NW>(wk, &as, kRec ? &unused : &qo, &lead);
         PT part = pzero_part(PT{});
         if (wk >= 0 && lead) {
           const V qv = first || probe ? as : fma(beta, qo, as);
@@ -763,8 +847,14 @@ __device__ bool cg_normal(const DevPlan& P, Team& tm, const BlockTabs& T, const 
       auto own_load = [&](int c, V* so, V* po, XT* xo) {
         int m = 0;
         if (coef_owner(P, c, wk, &m) && m < P.N) {
-          *so = ldcg(s + m);
-          if (!first) *po = ldcg(p + m);
+          if constexpr (kRec) {
+            *so = ldcg(s + m);
+            if (!first) *po = ldcg(p + m);
+          } else {
+            const V2 o = ldcg(sp + m);
+            *so = o.x;
+            *po = o.y;
+          }
           *xo = ldcg(x + m);
         }
       };
@@ -808,8 +898,12 @@ __device__ bool cg_normal(const DevPlan& P, Team& tm, const BlockTabs& T, const 
         if (wk >= 0 && lead) {
           const V pn = first ? so : fma(beta, po, so);
           const V sn = fma(-alpha, t, so);
-          stcg(s + m, sn);
-          stcg(p + m, pn);
+          if constexpr (kRec) {
+            stcg(s + m, sn);
+            stcg(p + m, pn);
+          } else {
+            stcg(sp + m, make_float2(sn, pn));
+          }
           stcg(x + m, static_cast<XT>(fma(static_cast<XT>(alpha), static_cast<XT>(pn), xo)));
           part = sq_part(sn, rs);
         }
@@ -859,8 +953,9 @@ template <int BT>
 __device__ bool pcg_normal_w(const DevPlan& P, Team& tm, const BlockTabs& T, double gamma0, double tol, int max_iter,
                              int stall, int* iters_out, double* gamma_out, int* status_out) {
   constexpr int NW = BT / 32 - 1;
-  __shared__ double2 wpart2[kUnitGroup][NW];
-  __shared__ double sh_ab[3];  // alpha, beta, final relative gamma
+  __shared__ float4 wpart2[kUnitGroup][NW];
+  __shared__ float sh_ab[2];   // alpha, beta
+  __shared__ double sh_gam;
   __shared__ int sh_ctl[2];    // stop flag, iterations
   *status_out = FCT_OK;
   *iters_out = 0;
@@ -873,8 +968,19 @@ __device__ bool pcg_normal_w(const DevPlan& P, Team& tm, const BlockTabs& T, dou
   const int wk = static_cast<int>(threadIdx.x) - 32;
   const int warp = static_cast<int>(threadIdx.x >> 5) - 1;
   const int lane32 = threadIdx.x & 31;
-  const double rs = 1.0 / sqrt(gamma0);
-  const double tol2 = tol * tol;
+  int e0 = 0;
+  frexp(gamma0, &e0);
+  const double rs = ldexp(1.0, -(e0 / 2));  // exact scaling near 1/sqrt(gamma0)
+  const float rsf = static_cast<float>(rs);
+  const float tol2 = static_cast<float>(tol * tol * (gamma0 * rs * rs));
+  // (r.r, w.r) of one element as double-float pairs, exact
+  auto products = [&](float r, float w) {
+    const float tr = r * rsf, tw = w * rsf;
+    const float2 rr = df_square(tr);
+    const float wr = __fmul_rn(tw, tr);
+    return make_float4(rr.x, rr.y, wr, fmaf(tw, tr, -wr));
+  };
+  float4* const pw = reinterpret_cast<float4*>(P.pw64);
   float* const wb0 = P.wv;
   float* const wb1 = P.wv + N;
   float* const vr = P.wv + 2 * static_cast<size_t>(N);
@@ -884,7 +990,8 @@ __device__ bool pcg_normal_w(const DevPlan& P, Team& tm, const BlockTabs& T, dou
   float* const vx = P.dx32;
   const float* const rhs = reinterpret_cast<const float*>(P.sp32);  // s, the first half
   // thread 0's state
-  double gam_prev = 1.0, al_prev = 1.0, best = 1.0e300, gam_last = 1.0;
+  float2 gam_prev = make_float2(1.0f, 0.0f), al_prev = gam_prev, gam_last = df_of(gamma0 * rs * rs);
+  float best = 3.0e38f;
   int best_it = 0;
 
   // y[m] = sum_j W[m][j] src[j * stride] for row m of unit u (k-th unit of this block)
@@ -925,12 +1032,11 @@ __device__ bool pcg_normal_w(const DevPlan& P, Team& tm, const BlockTabs& T, dou
     }
     return lane_group_sum((a0 + a1) + (a2 + a3), LW);
   };
-  auto warp_part2 = [&](int kk, double2 v) {
-    v.x = warp_sum(v.x);
-    v.y = warp_sum(v.y);
+  auto warp_part2 = [&](int kk, float4 v) {
+    v = warp_sum(v);
     if (wk >= 0 && lane32 == 0) wpart2[kk][warp] = v;
   };
-  auto flush2 = [&](double2* part, int u0, int nk) {
+  auto flush2 = [&](float4* part, int u0, int nk) {
     __syncthreads();
     if (threadIdx.x < nk) {
       stcg(part + u0 + threadIdx.x * tm.G, warps_sum<NW>(wpart2[threadIdx.x]));
@@ -946,30 +1052,29 @@ __device__ bool pcg_normal_w(const DevPlan& P, Team& tm, const BlockTabs& T, dou
       bool lead = false;
       float y = 0.0f;
       if (wk >= 0) y = gather(u, k, rhs, 1, &m, &lead);
-      double2 part = make_double2(0.0, 0.0);
+      float4 part = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
       if (wk >= 0 && lead) {
         const float r = ldcg(rhs + m);
         stcg(vr + m, r);
         stcg(wb0 + m, y);
         stcg(vx + m, 0.0f);
-        const double tr = r * rs, tw = y * rs;
-        part = make_double2(tr * tr, tw * tr);
+        part = products(r, y);
       }
       warp_part2(kg, part);
       if (++kg == kUnitGroup && u + tm.G < nwu) {
-        flush2(P.pw64, u0, kg);
+        flush2(pw, u0, kg);
         kg = 0;
         u0 = u + tm.G;
       }
     }
-    if (!phase_end<NW>(tm, wpart2, P.pw64, u0, kg)) return false;
+    if (!phase_end<NW>(tm, wpart2, pw, u0, kg)) return false;
   }
   int ctl = 0, it = 0;
   for (;; ++it) {
     const float* wcur = (it & 1) ? wb1 : wb0;
     float* wnext = (it & 1) ? wb0 : wb1;
-    const double2* pin = P.pw64 + ((it & 1) ? nwu : 0);
-    double2* pout = P.pw64 + ((it & 1) ? 0 : nwu);
+    const float4* pin = pw + ((it & 1) ? nwu : 0);
+    float4* pout = pw + ((it & 1) ? 0 : nwu);
     int u = tm.rank;
     int m = 0;
     bool lead = false;
@@ -990,55 +1095,59 @@ __device__ bool pcg_normal_w(const DevPlan& P, Team& tm, const BlockTabs& T, dou
         if (lead) own_load();
       }
     } else {
-      const double2 g = warp0_sum(pin, nwu);
+      const float4 g = warp0_sum(pin, nwu);
       if (threadIdx.x == 0) {
         int c = 0;
-        double al = 0.0, bt = 0.0;
-        const double gam = g.x, del = g.y;
+        float2 al = make_float2(0.0f, 0.0f), bt = al;
+        const float2 gam = make_float2(g.x, g.y), del = make_float2(g.z, g.w);
         gam_last = gam;
-        if (!isfinite(gam) || !isfinite(del)) {
+        if (!isfinite(gam.x) || !isfinite(del.x)) {
           c = FCT_ERR_NONFINITE + 16;
-        } else if (gam <= tol2) {
+        } else if (gam.x <= tol2) {
           c = 1;
         } else if (it >= max_iter) {
           c = FCT_ERR_NOCONV + 16;
         } else {
           if (stall > 0) {
-            if (gam < best) {
-              best = gam;
+            if (gam.x < best) {
+              best = gam.x;
               best_it = it;
             } else if (it - best_it >= stall) {
               c = 1;
             }
           }
           if (c == 0) {
-            bt = it == 0 ? 0.0 : gam / gam_prev;
-            const double den = it == 0 ? del : del - bt * gam / al_prev;
-            if (!(den > 0.0)) {
+            float2 den = del;
+            if (it > 0) {
+              bt = df_div(gam, gam_prev);
+              const float2 u = df_div(df_mul(bt, gam), al_prev);
+              den = df_add(del, make_float2(-u.x, -u.y));
+            }
+            if (!(den.x > 0.0f)) {
               c = 1;  // W is positive semidefinite: no further progress in this precision
             } else {
-              al = gam / den;
+              al = df_div(gam, den);
               gam_prev = gam;
               al_prev = al;
             }
           }
         }
-        sh_ab[0] = al;
-        sh_ab[1] = bt;
+        sh_ab[0] = al.x;
+        sh_ab[1] = bt.x;
         sh_ctl[0] = c;
       }
     }
     __syncthreads();
     ctl = sh_ctl[0];
     if (ctl != 0) break;
-    const float al = static_cast<float>(sh_ab[0]), bt = static_cast<float>(sh_ab[1]);
+    const float al = sh_ab[0], bt = sh_ab[1];
     int k = 0, kg = 0, u0 = u;
     for (; u < nwu; u += tm.G, ++k) {
       if (k > 0 && wk >= 0) {
         y = gather(u, k, wcur, 1, &m, &lead);
         if (lead) own_load();
       }
-      double2 part = make_double2(0.0, 0.0);
+      float4 part = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
       if (wk >= 0 && lead) {
         if (it == 0) {
           zv = y;
@@ -1058,8 +1167,7 @@ __device__ bool pcg_normal_w(const DevPlan& P, Team& tm, const BlockTabs& T, dou
         stcg(vx + m, xv);
         stcg(vr + m, r);
         stcg(wnext + m, wv);
-        const double tr = r * rs, tw = wv * rs;
-        part = make_double2(tr * tr, tw * tr);
+        part = products(r, wv);
       }
       warp_part2(kg, part);
       if (++kg == kUnitGroup && u + tm.G < nwu) {
@@ -1072,12 +1180,12 @@ __device__ bool pcg_normal_w(const DevPlan& P, Team& tm, const BlockTabs& T, dou
   }
   if (threadIdx.x == 0) {
     sh_ctl[1] = it;
-    sh_ab[2] = gam_last;
+    sh_gam = widen(gam_last);
   }
   __syncthreads();
   *status_out = ctl >= 16 ? ctl - 16 : FCT_OK;
   *iters_out = sh_ctl[1];
-  *gamma_out = sh_ab[2] * gamma0;
+  *gamma_out = sh_gam / (rs * rs);
   __syncthreads();
   return true;
 }
@@ -1087,8 +1195,11 @@ __device__ bool pcg_normal_w(const DevPlan& P, Team& tm, const BlockTabs& T, dou
 // nonempty bins, then the FP64 solve, or FP64 normal-residual sweeps around
 // FP32 inner solves (mixed).
 // ---------------------------------------------------------------------------
+// Inlined at each of the kernel's three call sites (alone, batch, serving): as a
+// function its tables and team would live in local memory, whose lines every
+// barrier's acquire drops (sparse D = 100, N = 50000: 62.0 ms against 56.9).
 template <int BT, bool SV, int DEEP>
-__device__ bool solve_job(const SolveJob& J, Team& tm, double* red, unsigned char* dsm, int smem_bytes) {
+__device__ __forceinline__ bool solve_job(const SolveJob& J, Team& tm, double* red, unsigned char* dsm, int smem_bytes) {
   // The plan's header in shared memory: every barrier's gpu-scope acquire drops
   // L1, so the first use after a barrier of a field held in global memory would
   // cost an L2 round trip, and a phase starts with a chain of them (D = 6 degree
@@ -1117,9 +1228,15 @@ __device__ bool solve_job(const SolveJob& J, Team& tm, double* red, unsigned cha
   }
   load_block_tabs<BT>(P, tm, dsm, smem_bytes, &T, J.precision == FCT_MIXED && P.n_w_units > 0 && P.s_init == nullptr,
                       SV ? (J.precision == FCT_MIXED ? 4 : 8) : 0, !cells);
-  // s and p of the CG solves are the halves of sp and sp32
+  // s and p of the CG solves: the halves of sp (FP64) and of sp32 (by grid groups
+  // and on W), or interleaved in sp32 (the two-matrix FP32 form)
   double* const s64 = reinterpret_cast<double*>(P.sp);
   float* const s32 = reinterpret_cast<float*>(P.sp32);
+  const bool interleaved = !cells && P.n_w_units == 0;
+  auto put_s32 = [&](int m, float v) {
+    if (interleaved) stcg(P.sp32 + m, make_float2(v, 0.0f));
+    else stcg(s32 + m, v);
+  };
   const int ncc = P.n_coef_chunks, nre = P.n_rowel_chunks, nru = P.n_row_units, nwide = P.n_wide_units;
   const int wk = static_cast<int>(threadIdx.x) - 32;
   const int nce = (P.N + BT - 1) / BT;  // elementwise units over coefficients
@@ -1186,7 +1303,7 @@ __device__ bool solve_job(const SolveJob& J, Team& tm, double* red, unsigned cha
   if (!isfinite(gamma0)) {
     status = FCT_ERR_NONFINITE;
   } else if (J.precision != FCT_MIXED) {
-    if (!cg_normal<BT, double, double, double, SV, DEEP>(P, tm, T, P.wcsr, P.wcm, s64, s64 + P.N, P.q, J.coeffs, gamma0, J.tol,
+    if (!cg_normal<BT, double, double, double, SV, DEEP>(P, tm, T, P.wcsr, P.wcm, s64, P.q, J.coeffs, gamma0, J.tol,
                                                J.max_iter, 0, &iters, &gfinal, &status, red))
       return false;
   } else if (gamma0 > 0.0) {
@@ -1198,7 +1315,7 @@ __device__ bool solve_job(const SolveJob& J, Team& tm, double* red, unsigned cha
     for (int u = tm.rank; u < nce; u += tm.G) {
       const int m = u * BT + threadIdx.x;
       if (m < P.N) {
-        stcg(s32 + m, static_cast<float>(ldcg(s64 + m) * ci));
+        put_s32(m, static_cast<float>(ldcg(s64 + m) * ci));
         stcg(P.dx32 + m, 0.0f);
       }
     }
@@ -1216,7 +1333,7 @@ __device__ bool solve_job(const SolveJob& J, Team& tm, double* red, unsigned cha
           if (!cg_cells<BT>(P, tm, dsm, g64 * ci * ci, J.inner_tol, J.max_iter, 64, &it_in, &g_in, &st_in))
             return false;
         }
-      } else if (!cg_normal<BT, float, float, float, SV, DEEP>(P, tm, T, P.wcsr32, P.wcm32, s32, s32 + P.N, P.q32, P.dx32,
+      } else if (!cg_normal<BT, float, float, float, SV, DEEP>(P, tm, T, P.wcsr32, P.wcm32, s32, P.q32, P.dx32,
                                                      g64 * ci * ci, J.inner_tol, J.max_iter, 64, &it_in, &g_in,
                                                      &st_in, red)) {
         return false;
@@ -1254,7 +1371,7 @@ __device__ bool solve_job(const SolveJob& J, Team& tm, double* red, unsigned cha
         t = coef_combine<BT / 32 - 1>(P, T, t, kc, wk, m, &lead);
         double part = 0.0;
         if (lead) {
-          stcg(s32 + m, static_cast<float>(t * ci));
+          put_s32(m, static_cast<float>(t * ci));
           stcg(s64 + m, t);  // for an FP64 continuation
           stcg(P.dx32 + m, 0.0f);
           part = t * t;
@@ -1278,7 +1395,7 @@ __device__ bool solve_job(const SolveJob& J, Team& tm, double* red, unsigned cha
         int it64 = 0, st64 = FCT_OK;
         double g_out = g64;
         const double tol_eff = J.tol * sqrt(gamma0 / g64);
-        if (!cg_normal<BT, double, double, double, SV, DEEP>(P, tm, T, P.wcsr, P.wcm, s64, s64 + P.N, P.q, x, g64, tol_eff, J.max_iter,
+        if (!cg_normal<BT, double, double, double, SV, DEEP>(P, tm, T, P.wcsr, P.wcm, s64, P.q, x, g64, tol_eff, J.max_iter,
                                                    0, &it64, &g_out, &st64, red))
           return false;
         iters += it64;
