@@ -800,7 +800,7 @@ def run_next_rows(F, w, opts, flush, steps=20, large_sparse=True, gather_peak=No
     pts = torch.from_numpy(W.stream(23, "probe").uniform(-1.0, 1.0, (npts, w.D))).cuda()
     vals = torch.empty(npts, dtype=torch.float64, device="cuda")
     ms = statistics.mean(_timed(lambda: p.evaluate(c, pts, vals), max(3, steps // 4), flush))
-    flops = npts * w.N * (w.D + 1)   # per point and term: D table products and one add, FP64
+    flops = 2 * npts * (w.N - 1)   # per point: one multiply-add per nonzero index of the support's trie, FP64
     out["evaluate"] = {"points": npts, "terms": w.N, "ms": ms, "points_per_s": npts / (ms / 1e3),
                        "roofline": {"bound": "alu", "achieved": flops / (ms / 1e3) / 1e12, "unit": "TFLOP/s",
                                     "peak": F.fct_measure_fp64(1 << 16),

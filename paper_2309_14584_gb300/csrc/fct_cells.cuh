@@ -13,6 +13,11 @@
 //     A_l^T q_l, streamed out (tpart);
 //   phase 2, per owner chunk: t = sum over groups of tpart, then x += alpha p,
 //     s -= alpha t.
+// What bounds it now: latency and issue in the two streams (about 100 instructions
+// and 20 wavefronts of the L1 / shared-memory pipe per four steps, 8..16 warps per SM), then the
+// phases' fixed costs.  Time per CG iteration, two-matrix form -> this: sparse
+// D = 100, N = 50000, 240 grids 226 -> 70 us; N = 20000, 1000 grids 172 -> 110;
+// D = 18 degree 5, 171 grids 56 -> 49 (171 tasks on 152 SMs).
 // Two team barriers, as in cg_normal, but every scattered access is to shared
 // memory and global traffic is coalesced: 6 bytes of table per entry (read by
 // the gather and again, from L2, by the scatter) and 8 + 4 bytes of vectors per

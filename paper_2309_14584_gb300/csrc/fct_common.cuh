@@ -126,8 +126,10 @@ __device__ __forceinline__ double pzero(double) { return 0.0; }
 // hi + lo (hi = v v rounded, lo = fma(v, v, -hi)), and pairs are added with
 // Knuth's two-sum, so a warp's sum carries about 48 significant bits.  GB300
 // runs FP64 at a small fraction of its FP32 rate, so the FP32 inner solves
-// form their inner products this way and convert each warp's pair to FP64
-// once per group of units (widen); sums across warps and units are FP64.
+// form their inner products this way, sums across warps and units and the
+// scalars alpha and beta included (an FP64 quotient by one thread between two
+// team barriers took about 0.8 us: D = 6 degree 10 mixed 1.00 -> 0.89 ms with the
+// plan's header in shared memory).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ float2 df_two_sum(float a, float b) {
   const float s = a + b;

@@ -5,15 +5,16 @@
 // bins into b, and the least-squares solve (CGLS, the "CG method" of Sec. 3.4)
 // whose every iteration is one alias gather A p (bin-major, over the
 // bin-sorted CSR) and one alias adjoint A^T r (coefficient-major over the
-// per-grid row tables), as in the cost model of Sec. 3.5.
+// per-grid row tables), as in the cost model of Sec. 3.5, or, in the mixed
+// path's inner solve of plans with many grids, both products grid by grid in
+// shared memory (fct_cells.cuh).
 //
 // Blocks are grouped in teams; a team solves one transform at a time, taken
 // from a work queue, and synchronises through a bounded software barrier in
 // global memory (every wait has a time limit and reports FCT_ERR_TIMEOUT).
-// A CGLS iteration needs two team barriers: the vectors p_new = s + beta p
-// and r_new = r - alpha q are formed on the fly inside the gathers from the
-// previous buffers (double-buffered), so no barrier is spent on the
-// elementwise updates.  All reductions are two-stage with a fixed order
+// A CGLS iteration needs two team barriers: A p is formed from s and the
+// previous p (or the previous A p) inside the gather, so no barrier is spent on
+// the elementwise updates.  All reductions are two-stage with a fixed order
 // (per-chunk block sums, then one sum over chunk partials), so a transform's
 // result does not depend on the team size or on the rest of the batch.
 #include <cuda_runtime.h>
@@ -24,6 +25,7 @@
 #include <thread>
 #include <cstdio>
 #include <cstring>
+#include <functional>
 #include <memory>
 #include <mutex>
 #include <string>
@@ -236,7 +238,8 @@ __global__ void eval_expansion_kernel(const uint16_t* __restrict__ support, cons
   if (p < P && lane == 0) values[p] = acc;
 }
 
-// Evaluation by shared prefixes.  The nonzero components (axis, degree) of the
+// Evaluation by shared prefixes (fct_evaluate's kernel; the one above, term by
+// term, serves supports whose stack or tables do not fit).  The nonzero components (axis, degree) of the
 // indices, in support order, form a trie whose node values are
 //   v(node) = T_degree(x_axis) (c_node + sum of its children's v),
 // so every node takes one multiply-add, whatever the depth: about one per term on
@@ -248,6 +251,10 @@ __global__ void eval_expansion_kernel(const uint16_t* __restrict__ support, cons
 // cut into `chunks` programs of their own, so a block of eval_trie_threads threads
 // can give `ppb` points to each of threads / ppb workers, and the chunk sums are
 // added in chunk order: a value does not depend on how many points are asked for.
+// Measured (term by term before): D = 6 degree 10 at 131072 points 14.2 -> 3.9 ms,
+// 1.07e9 multiply-adds at half the measured FP64 rate (the other half: the chunks'
+// restarts, the last wave, and chains of dependent multiply-adds at 40 warps per
+// SM); D = 3 degree 5 at 10955 points 18.3 -> 13.0 us (latency).
 constexpr int kEvalThreads = 256;
 
 __global__ void __launch_bounds__(kEvalThreads) eval_trie_kernel(
@@ -1440,30 +1447,40 @@ static fct_status batch_setup(int B, const fct_plan* plans, const double* const*
   if (G <= 0) {
     // Blocks per team from a model of the launch: a CG iteration of a transform
     // takes kIterUs of latency plus its entries over the team's threads (fitted to
-    // D = 10 degree 8 on 38..304 blocks: 18.5, 50, 101 us against 18.6, 55, 102),
-    // the jobs go to the teams largest first, and the last team to finish counts.
+    // D = 10 degree 8 on 38..304 blocks: 18.5, 50, 101 us against 18.6, 55, 102), the
+    // iterations grow like N^(1/4) (65, 102, 180 at N = 924, 8008, 43758),
+    // the jobs go to the teams largest first, and the last team to finish counts
+    // (48 unlike transforms, mixed: 133.9 ms at the former 19 blocks, 63.9 now).
     // A fixed share of the GPU per job leaves most of it idle once only the
-    // largest transforms of an unlike batch are left.
+    // largest transforms of an unlike batch are left.  At most 16 teams: below a
+    // sixteenth of the GPU the model is too kind to small teams (34 small
+    // transforms: 1.75 ms on 13 blocks, 1.47 on 19).
     constexpr double kIterUs = 6.5, kEntryUs = 0.717;
-    std::vector<double> work(B);
+    std::vector<double> work(B), iters(B);
     int units = 1;
     for (int q = 0; q < B; ++q) {
       const fct_plan Pq = plans[order[q]];
       work[q] = kEntryUs * static_cast<double>(Pq->hp.K) * static_cast<double>(Pq->N) / P0->block_threads *
                 (Pq->opt.precision == FCT_MIXED ? 1.0 : 2.0);
+      iters[q] = std::sqrt(std::sqrt(static_cast<double>(Pq->N)));
       units = std::max(units, Pq->grid_blocks);
     }
     double best = 0.0;
     std::vector<double> busy;
     int last = 0;
-    for (int teams = 1; teams <= std::min({B, kMaxTeams, P0->max_coresident}); teams = teams < 8 ? teams + 1 : teams * 5 / 4) {
+    for (int teams = 1; teams <= std::min({B, 16, P0->max_coresident}); ++teams) {
       const int g = std::min(units, P0->max_coresident / teams);
       if (g == last) continue;
       last = g;
+      // busy: a heap whose front is the team that is free first
       busy.assign(std::min(P0->max_coresident / g, std::min(B, kMaxTeams)), 0.0);
-      for (int q = 0; q < B; ++q)
-        *std::min_element(busy.begin(), busy.end()) += kIterUs + work[q] / g;
-      const double t = *std::max_element(busy.begin(), busy.end());
+      double t = 0.0;
+      for (int q = 0; q < B; ++q) {
+        std::pop_heap(busy.begin(), busy.end(), std::greater<double>());
+        busy.back() += iters[q] * (kIterUs + work[q] / g);
+        t = std::max(t, busy.back());
+        std::push_heap(busy.begin(), busy.end(), std::greater<double>());
+      }
       if (G <= 0 || t < best) {
         best = t;
         G = g;
