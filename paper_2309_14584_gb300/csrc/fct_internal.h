@@ -431,13 +431,15 @@ struct CellLayout {
 // 18 in the two-matrix form), and enough coefficients and entries that the work
 // outweighs its phases' longer latency (D = 60, N = 5027, 637 grids: 48 us against
 // 39; D = 30, N = 6371, 202 grids: 30 against 42; D = 100, N = 50000, 240 grids:
-// 72 against 226).
+// 72 against 226), in at most kCellMaxSlices slices (N = 10^6, 600 grids, over 60
+// slices: 20.9 s a transform against 20.3, and 10 GB of tables).
 constexpr int64_t kCellMinN = 6144;
 constexpr int64_t kCellMinEntries = int64_t{1} << 20;
 bool cells_pay(int64_t N, int K, int block_threads, int64_t wave);
 constexpr int kCellRun = 64;          // longest run of a row
 constexpr int kCellIdle = 5;          // idle groups after a cell's last (destinations read ahead)
 constexpr int kCellFew = 8;           // runs of a row that one thread adds up
+constexpr int kCellMaxSlices = 8;
 constexpr int kCellMaxSlice = 32736;  // 15-bit coefficient index, 32 padding slots included
 // Chooses the layout from the rows of every grid (L->rows), the block size,
 // the co-resident blocks `wave`, the shared memory `cap` a block may take and

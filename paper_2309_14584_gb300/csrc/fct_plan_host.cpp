@@ -570,7 +570,7 @@ void choose_cells(int64_t N, int K, int64_t M, int block_threads, int64_t wave, 
     if (sl < std::min<int64_t>(ncap, 2048)) continue;
     const int64_t S = (N + sl - 1) / sl;
     sl = ((N + S - 1) / S + 31) / 32 * 32;
-    if ((S - 1) * sl >= N) continue;
+    if ((S - 1) * sl >= N || S > kCellMaxSlices) continue;
     const int64_t NG = (K + gg - 1) / gg, np = S * sl;
     const int64_t ext = 2 * (sl / kCellRun) + 2;
     int64_t qmax = 0;
