@@ -1,7 +1,7 @@
 """Build the in-tree CUDA library libfct_gb300.so for sm_103a with nvcc.
 
 The translation units (host tables, the library's host code and small
-kernels, and one per block size for the team solver kernels) are compiled in
+kernels, and three per block size for the team solver kernels) are compiled in
 parallel and linked into one shared library (static CUDA runtime), next to
 this file.  No torch headers are used:
 the library's ABI is plain C (include/fct.h).
@@ -21,8 +21,8 @@ BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libfct_gb300.so")
 
 SOURCES = ["fct_solve_k256.cu", "fct_solve_k128.cu", "fct_solve_k512.cu", "fct_solve_k256d.cu", "fct_solve_k128d.cu",
-           "fct_solve_k512d.cu", "fct_device.cu", "fct_plan_device.cu", "fct_plan_host.cpp", "fct_peaks.cu",
-           "fct_dct_tc.cu"]
+           "fct_solve_k512d.cu", "fct_solve_k256c.cu", "fct_solve_k128c.cu", "fct_solve_k512c.cu", "fct_device.cu",
+           "fct_plan_device.cu", "fct_plan_host.cpp", "fct_peaks.cu", "fct_dct_tc.cu"]
 HEADERS = ["fct_internal.h", "fct_common.cuh", "fct_solver.cuh", "fct_cells.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

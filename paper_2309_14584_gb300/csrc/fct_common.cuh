@@ -400,9 +400,14 @@ __device__ __forceinline__ void st_release_sys_i32(int* p, int v) {
 
 
 // The team solver kernel (defined in fct_solver.cuh, instantiated per block
-// size in fct_solve_k128.cu, fct_solve_k256.cu and fct_solve_k512.cu).
+// size in fct_solve_k128*.cu, fct_solve_k256*.cu and fct_solve_k512*.cu).
+// SV: the CG loop's entry values are staged in shared memory too.
 // DEEP = 1: the gathers stage twice as many entries per lane and round (8
 // per row lane, 16 per coefficient lane), for plans with long rows or many
 // grids, whose gathers stream their tables from DRAM.
-template <int BT, bool SV, int DEEP>
+// CELLS: the launch may hold plans whose inner solve runs by grid groups
+// (fct_cells.cuh).  A variant of its own: with that solve in every variant the
+// others spilled (256 threads, plain: 952 bytes of spill stores, none now; 38
+// transforms of D = 6 degree 10, mixed, on 16-block teams: 31.2 ms, 28.0 now).
+template <int BT, bool SV, int DEEP, bool CELLS>
 __global__ void __launch_bounds__(BT, 512 / BT) fct_solve_kernel(const SolveArgs a);

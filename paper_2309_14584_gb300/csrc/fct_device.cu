@@ -368,6 +368,7 @@ struct fct_plan_s {
   int blocks_per_sm = 1;
   int smem_bytes = 0;          // dynamic shared memory requested per block
   int smem_cap = 0;            // largest request that keeps blocks_per_sm resident
+  int cells_cap = 0;           // the same for the variant with the inner solve by grid groups
   std::vector<int32_t> ru_first, rowptr_h;  // for the shared-memory sizing of other team sizes
   std::vector<int32_t> w_rowptr_h;          // row pointer of W = A^T A (empty when not built)
   bool stage_values = false;                // single launches stage the CG loop's entry values too
@@ -402,14 +403,17 @@ fct_status cuda_fail(cudaError_t e, const char* what) {
 // CG loop's entry values in shared memory (single transforms whose tables
 // fit); kKernelDeep stages twice as many gather entries per lane and round
 // (single transforms of plans with wide rows or many grids, whose tables
-// stream from DRAM).  See choose_shape.
-enum { kKernelPlain = 0, kKernelStaged = 1, kKernelDeep = 2 };
+// stream from DRAM); kKernelCells is the plain one with the inner solve by grid
+// groups (plans that solve so, batches that hold one, servers).  See
+// choose_shape.
+enum { kKernelPlain = 0, kKernelStaged = 1, kKernelDeep = 2, kKernelCells = 3 };
 
 template <int BT>
 const void* kernel_ptr(int kind) {
-  if (kind == kKernelStaged) return reinterpret_cast<const void*>(&fct_solve_kernel<BT, true, 0>);
-  if (kind == kKernelDeep) return reinterpret_cast<const void*>(&fct_solve_kernel<BT, false, 1>);
-  return reinterpret_cast<const void*>(&fct_solve_kernel<BT, false, 0>);
+  if (kind == kKernelStaged) return reinterpret_cast<const void*>(&fct_solve_kernel<BT, true, 0, false>);
+  if (kind == kKernelDeep) return reinterpret_cast<const void*>(&fct_solve_kernel<BT, false, 1, false>);
+  if (kind == kKernelCells) return reinterpret_cast<const void*>(&fct_solve_kernel<BT, false, 0, true>);
+  return reinterpret_cast<const void*>(&fct_solve_kernel<BT, false, 0, false>);
 }
 
 const void* solve_kernel_for(int bt, int kind = kKernelPlain) {
@@ -481,29 +485,33 @@ size_t launch_smem(const fct_plan P, int G, size_t cap) {
 }
 
 // Dynamic shared memory a solver block may take without lowering the blocks
-// per SM of the plain kernel (the largest static shared memory of the
-// kernel variants counted), set as every variant's limit.  Plans and servers
-// of one block size compute the same value, so neither lowers the other's
-// launch limit.
-fct_status solver_smem_cap(int bt, const cudaDeviceProp& prop, int* cap_out, int* per_sm_out) {
-  const void* kfn = solve_kernel_for(bt);
-  cudaFuncAttributes fa;
-  FCT_CUDA(cudaFuncGetAttributes(&fa, kfn));
-  for (int kind : {kKernelStaged, kKernelDeep}) {
+// per SM of the plain kernel, set as the variants' limit: one value for the
+// variants without the inner solve by grid groups (the largest static shared
+// memory among them counted), at most as much for the one with it.  Plans and
+// servers of one block size compute the same values, so neither lowers the
+// other's launch limit.
+fct_status solver_smem_cap(int bt, const cudaDeviceProp& prop, int* cap_out, int* cells_cap_out, int* per_sm_out) {
+  int per_sm = 0;
+  FCT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, solve_kernel_for(bt), bt, 0));
+  if (per_sm < 1) return fail(FCT_ERR_CUDA, "solver kernel cannot be resident");
+  size_t fixed[4];
+  for (int kind : {kKernelPlain, kKernelStaged, kKernelDeep, kKernelCells}) {
     cudaFuncAttributes fk;
     FCT_CUDA(cudaFuncGetAttributes(&fk, solve_kernel_for(bt, kind)));
-    fa.sharedSizeBytes = std::max(fa.sharedSizeBytes, fk.sharedSizeBytes);
+    fixed[kind] = fk.sharedSizeBytes;
   }
-  int per_sm = 0;
-  FCT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kfn, bt, 0));
-  if (per_sm < 1) return fail(FCT_ERR_CUDA, "solver kernel cannot be resident");
-  const int reserve = 1024;  // per-block system reservation
-  int cap = static_cast<int>(prop.sharedMemPerMultiprocessor / per_sm) - reserve - static_cast<int>(fa.sharedSizeBytes);
-  cap = std::min(cap, static_cast<int>(prop.sharedMemPerBlockOptin) - static_cast<int>(fa.sharedSizeBytes));
-  cap = std::max(cap, 0) & ~15;
-  for (int kind : {kKernelPlain, kKernelStaged, kKernelDeep})
-    FCT_CUDA(cudaFuncSetAttribute(solve_kernel_for(bt, kind), cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
-  *cap_out = cap;
+  auto cap_for = [&](size_t sh) {
+    const int reserve = 1024;  // per-block system reservation
+    int cap = static_cast<int>(prop.sharedMemPerMultiprocessor / per_sm) - reserve - static_cast<int>(sh);
+    cap = std::min(cap, static_cast<int>(prop.sharedMemPerBlockOptin) - static_cast<int>(sh));
+    return std::max(cap, 0) & ~15;
+  };
+  const size_t plain = std::max({fixed[kKernelPlain], fixed[kKernelStaged], fixed[kKernelDeep]});
+  *cap_out = cap_for(plain);
+  *cells_cap_out = cap_for(std::max(plain, fixed[kKernelCells]));
+  for (int kind : {kKernelPlain, kKernelStaged, kKernelDeep, kKernelCells})
+    FCT_CUDA(cudaFuncSetAttribute(solve_kernel_for(bt, kind), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  kind == kKernelCells ? *cells_cap_out : *cap_out));
   *per_sm_out = per_sm;
   return FCT_OK;
 }
@@ -528,13 +536,15 @@ CellBytes cell_bytes(const CellLayout& L, int K) {
 // L->rows filled in.
 fct_status choose_cell_layout(fct_plan P, int64_t wave, CellLayout* L) {
   if (!cells_pay(P->N, P->K, P->block_threads, wave)) return FCT_OK;  // before the device is asked
-  int dev = 0, cap = 0, per_sm = 0;
+  int dev = 0, cap = 0, cells_cap = 0, per_sm = 0, cells_per_sm = 0;
   FCT_CUDA(cudaGetDevice(&dev));
   cudaDeviceProp prop;
   FCT_CUDA(cudaGetDeviceProperties(&prop, dev));
-  const fct_status s = solver_smem_cap(P->block_threads, prop, &cap, &per_sm);
+  const fct_status s = solver_smem_cap(P->block_threads, prop, &cap, &cells_cap, &per_sm);
   if (s != FCT_OK) return s;
-  choose_cells(P->N, P->K, P->M, P->block_threads, wave, cap, L);
+  FCT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+      &cells_per_sm, solve_kernel_for(P->block_threads, kKernelCells), P->block_threads, cells_cap));
+  if (cells_per_sm >= per_sm) choose_cells(P->N, P->K, P->M, P->block_threads, wave, cells_cap, L);
   return FCT_OK;
 }
 
@@ -544,14 +554,15 @@ fct_status choose_shape(fct_plan P) {
   cudaDeviceProp prop;
   FCT_CUDA(cudaGetDeviceProperties(&prop, dev));
   if (!prop.cooperativeLaunch) return fail(FCT_ERR_CUDA, "device does not support cooperative launch");
-  const void* kfn = solve_kernel_for(P->block_threads);
-  int cap = 0, per_sm = 0;
-  const fct_status cs = solver_smem_cap(P->block_threads, prop, &cap, &per_sm);
+  const bool cells = P->hp.tk_groups > 0;
+  const void* kfn = solve_kernel_for(P->block_threads, cells ? kKernelCells : kKernelPlain);
+  int per_sm = 0;
+  const fct_status cs = solver_smem_cap(P->block_threads, prop, &P->smem_cap, &P->cells_cap, &per_sm);
   if (cs != FCT_OK) return cs;
+  const int cap = cells ? P->cells_cap : P->smem_cap;
   if (P->hp.coef_split && cap < coef_combine_bytes(P->block_threads))
     return fail(FCT_ERR_CUDA, "no shared memory for the grid-split gather");
   P->blocks_per_sm = per_sm;
-  P->smem_cap = cap;
   P->max_coresident = per_sm * prop.multiProcessorCount;
   int units = std::max({P->hp.n_row_units, P->hp.n_coef_chunks, P->hp.n_rowel_chunks, 1});
   for (int p = 0; p < P->H.npass; ++p)
@@ -564,7 +575,7 @@ fct_status choose_shape(fct_plan P) {
   const size_t need_values = team_smem_need(P, P->grid_blocks, true);
   // (plans whose inner solve runs by grid groups read the row tables in the
   // three FP64 sweeps only)
-  P->stage_values = need_values <= static_cast<size_t>(cap) && P->hp.tk_groups == 0;
+  P->stage_values = need_values <= static_cast<size_t>(cap) && !cells;
   P->smem_bytes = static_cast<int>((P->stage_values ? need_values : launch_smem(P, P->grid_blocks, cap)) + 15) & ~15;
   P->smem_bytes = std::min(P->smem_bytes, cap);
   int chk = 0;
@@ -575,8 +586,8 @@ fct_status choose_shape(fct_plan P) {
                                                            P->block_threads, P->smem_bytes));
     if (chk * prop.multiProcessorCount < P->grid_blocks) P->stage_values = false;
   }
-  P->kernel_kind = P->stage_values ? kKernelStaged : kKernelPlain;
-  if (!P->stage_values && (P->hp.n_wide_units > 0 || P->K >= 64)) {
+  P->kernel_kind = cells ? kKernelCells : P->stage_values ? kKernelStaged : kKernelPlain;
+  if (!cells && !P->stage_values && (P->hp.n_wide_units > 0 || P->K >= 64)) {
     FCT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&chk, solve_kernel_for(P->block_threads, kKernelDeep),
                                                            P->block_threads, P->smem_bytes));
     if (chk * prop.multiProcessorCount >= P->grid_blocks) P->kernel_kind = kKernelDeep;
@@ -1420,10 +1431,12 @@ fct_status fct_execute_host(fct_plan P, const double* samples_host, double* coef
 
 // Checks a batch, orders its jobs (largest transforms first: the shortest
 // tail for the device work queue) with each job's report at reports + i, and
-// fixes the launch shape: blocks per team G, teams, dynamic shared memory.
+// fixes the launch shape: blocks per team G, teams, dynamic shared memory, and
+// the kernel variant (the one with the inner solve by grid groups only if a
+// plan of the batch takes it).
 static fct_status batch_setup(int B, const fct_plan* plans, const double* const* samples, double* const* coeffs,
                               int team_blocks, fct_report* reports, std::vector<SolveJob>* jobs, int* G_out,
-                              int* teams_out, int* smem_out) {
+                              int* teams_out, int* smem_out, int* kind_out) {
   if (B < 1 || !plans || !samples || !coeffs) return fail(FCT_ERR_INVALID_ARG, "bad batch arguments");
   for (int i = 0; i < B; ++i) {
     if (!plans[i] || !samples[i] || !coeffs[i]) return fail(FCT_ERR_INVALID_ARG, "NULL plan or buffer in batch");
@@ -1490,9 +1503,13 @@ static fct_status batch_setup(int B, const fct_plan* plans, const double* const*
   G = std::min(G, P0->max_coresident);
   *teams_out = std::min(std::max(1, P0->max_coresident / G), std::min(B, kMaxTeams));
   *G_out = G;
+  *kind_out = kKernelPlain;
+  for (int i = 0; i < B; ++i)
+    if (plans[i]->hp.tk_groups > 0) *kind_out = kKernelCells;
+  const int cap = *kind_out == kKernelCells ? P0->cells_cap : P0->smem_cap;
   size_t need = 0;
-  for (int i = 0; i < B; ++i) need = std::max(need, launch_smem(plans[i], G, static_cast<size_t>(P0->smem_cap)));
-  *smem_out = std::min(static_cast<int>(std::min<size_t>(need, P0->smem_cap) + 15) & ~15, P0->smem_cap);
+  for (int i = 0; i < B; ++i) need = std::max(need, launch_smem(plans[i], G, static_cast<size_t>(cap)));
+  *smem_out = std::min(static_cast<int>(std::min<size_t>(need, cap) + 15) & ~15, cap);
   return FCT_OK;
 }
 
@@ -1514,8 +1531,8 @@ fct_status fct_execute_batch(int B, const fct_plan* plans, const double* const* 
   }
   fct_report* dreps = reinterpret_cast<fct_report*>(P0->djobs + P0->djobs_cap);
   std::vector<SolveJob> jobs;
-  int G = 0, teams = 0, smem = 0;
-  fct_status s = batch_setup(B, plans, samples, coeffs, team_blocks, dreps, &jobs, &G, &teams, &smem);
+  int G = 0, teams = 0, smem = 0, kind = kKernelPlain;
+  fct_status s = batch_setup(B, plans, samples, coeffs, team_blocks, dreps, &jobs, &G, &teams, &smem, &kind);
   if (s != FCT_OK) return s;
   FCT_CUDA(cudaMemcpyAsync(P0->djobs, jobs.data(), sizeof(SolveJob) * B, cudaMemcpyHostToDevice, st));
   FCT_CUDA(cudaStreamSynchronize(st));
@@ -1526,7 +1543,7 @@ fct_status fct_execute_batch(int B, const fct_plan* plans, const double* const* 
   a.ls = P0->ls;
   a.timeout_ns = timeout_ns(P0);
   a.smem_bytes = smem;
-  s = launch_solve(P0, a, teams * G, st);
+  s = launch_solve(P0, a, teams * G, st, kind);
   if (s != FCT_OK) return s;
   if (reps) return read_report(P0, dreps, st, reps, B);
   return FCT_OK;
@@ -1535,7 +1552,7 @@ fct_status fct_execute_batch(int B, const fct_plan* plans, const double* const* 
 }  // extern "C"
 
 struct fct_batch_s {
-  int B = 0, G = 0, teams = 0, smem = 0, block_threads = 0, device = 0;
+  int B = 0, G = 0, teams = 0, smem = 0, kind = 0, block_threads = 0, device = 0;
   unsigned long long tns = 0;
   SolveJob* djobs = nullptr;   // [B] jobs, then [B] reports
   fct_report* dreps = nullptr;
@@ -1564,7 +1581,8 @@ fct_status fct_batch_create(fct_batch* out, int B, const fct_plan* plans, const 
   e = cudaMemset(Bt->dreps, 0, sizeof(fct_report) * B);
   if (e != cudaSuccess) return fail_free(cuda_fail(e, "fct_batch_create"));
   std::vector<SolveJob> jobs;
-  fct_status s = batch_setup(B, plans, samples, coeffs, team_blocks, Bt->dreps, &jobs, &Bt->G, &Bt->teams, &Bt->smem);
+  fct_status s = batch_setup(B, plans, samples, coeffs, team_blocks, Bt->dreps, &jobs, &Bt->G, &Bt->teams, &Bt->smem,
+                             &Bt->kind);
   if (s != FCT_OK) return fail_free(s);
   e = cudaMemcpy(Bt->djobs, jobs.data(), sizeof(SolveJob) * B, cudaMemcpyHostToDevice);
   if (e != cudaSuccess) return fail_free(cuda_fail(e, "fct_batch_create"));
@@ -1600,7 +1618,7 @@ fct_status fct_batch_launch(fct_batch Bt, void* stream) {
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   void* kargs[] = {&a};
-  FCT_CUDA(cudaLaunchKernelExC(&cfg, solve_kernel_for(Bt->block_threads), kargs));
+  FCT_CUDA(cudaLaunchKernelExC(&cfg, solve_kernel_for(Bt->block_threads, Bt->kind), kargs));
   return FCT_OK;
 }
 
@@ -1684,6 +1702,7 @@ fct_status fct_plan_clone(fct_plan* out, fct_plan src) {
   C->stage_values = src->stage_values;
   C->kernel_kind = src->kernel_kind;
   C->smem_cap = src->smem_cap;
+  C->cells_cap = src->cells_cap;
   C->ru_first = src->ru_first;
   C->rowptr_h = src->rowptr_h;
   C->w_rowptr_h = src->w_rowptr_h;
@@ -1873,8 +1892,9 @@ extern "C" fct_status fct_execute_noalloc(fct_plan P, const double* samples, dou
   a.timeout_ns = timeout_ns(P);
   a.smem_bytes = P->smem_bytes;
   void* kargs[] = {&a};
-  FCT_CUDA(cudaLaunchCooperativeKernel(solve_kernel_for(P->block_threads), dim3(P->grid_blocks),
-                                       dim3(P->block_threads), kargs, static_cast<size_t>(a.smem_bytes), st));
+  FCT_CUDA(cudaLaunchCooperativeKernel(
+      solve_kernel_for(P->block_threads, P->hp.tk_groups > 0 ? kKernelCells : kKernelPlain), dim3(P->grid_blocks),
+      dim3(P->block_threads), kargs, static_cast<size_t>(a.smem_bytes), st));
   if (!rep) return FCT_OK;
   FCT_CUDA(cudaMemcpyAsync(rep, drep, sizeof(fct_report), cudaMemcpyDeviceToHost, st));
   int err = 0;
@@ -2038,8 +2058,11 @@ fct_status server_ensure_running(fct_server S) {
   a.ring = S->d_ring;
   a.idle_ns = S->idle_ns;
   void* kargs[] = {&a};
-  FCT_CUDA(cudaLaunchCooperativeKernel(solve_kernel_for(S->block_threads), dim3(S->teams * S->team_blocks),
-                                       dim3(S->block_threads), kargs, static_cast<size_t>(S->smem_bytes), S->stream));
+  // plans of either inner solve may be submitted while the launch runs, so it is
+  // the variant with both
+  FCT_CUDA(cudaLaunchCooperativeKernel(solve_kernel_for(S->block_threads, kKernelCells),
+                                       dim3(S->teams * S->team_blocks), dim3(S->block_threads), kargs,
+                                       static_cast<size_t>(S->smem_bytes), S->stream));
   FCT_CUDA(cudaEventRecord(S->done_ev, S->stream));
   S->launched = true;
   return FCT_OK;
@@ -2056,14 +2079,14 @@ fct_status fct_server_create(fct_server* out, int block_threads, int team_blocks
   if (block_threads != 128 && block_threads != 256 && block_threads != 512)
     return fail(FCT_ERR_INVALID_ARG, "block_threads must be 128, 256 or 512");
   if (!(idle_timeout_s > 0.0) || idle_timeout_s > 1.0) return fail(FCT_ERR_INVALID_ARG, "idle_timeout_s must be in (0, 1]");
-  int dev = 0, nsm = 0, per_sm = 0, cap = 0;
+  int dev = 0, nsm = 0, per_sm = 0, cap = 0, cells_cap = 0;
   FCT_CUDA(cudaGetDevice(&dev));
   FCT_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
   cudaDeviceProp prop;
   FCT_CUDA(cudaGetDeviceProperties(&prop, dev));
-  const fct_status cs = solver_smem_cap(block_threads, prop, &cap, &per_sm);
+  const fct_status cs = solver_smem_cap(block_threads, prop, &cap, &cells_cap, &per_sm);
   if (cs != FCT_OK) return cs;
-  if (cap < coef_combine_bytes(block_threads)) return fail(FCT_ERR_CUDA, "no shared memory for the solver");
+  if (cells_cap < coef_combine_bytes(block_threads)) return fail(FCT_ERR_CUDA, "no shared memory for the solver");
   const int coresident = per_sm * nsm;
   if (team_blocks <= 0) team_blocks = 16;
   team_blocks = std::min(team_blocks, coresident);
@@ -2074,7 +2097,7 @@ fct_status fct_server_create(fct_server* out, int block_threads, int team_blocks
   S->block_threads = block_threads;
   S->team_blocks = team_blocks;
   S->teams = teams;
-  S->smem_bytes = cap;
+  S->smem_bytes = cells_cap;
   S->idle_ns = static_cast<unsigned long long>(idle_timeout_s * 1e9);
   cudaError_t e = cudaHostAlloc(&S->h_ring, sizeof(ServerRing), cudaHostAllocMapped | cudaHostAllocPortable);
   if (e == cudaSuccess) {

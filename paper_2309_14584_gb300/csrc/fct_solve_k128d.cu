@@ -3,4 +3,4 @@
 // that the library's kernels build in parallel.
 #include "fct_solver.cuh"
 
-template __global__ void fct_solve_kernel<128, false, 1>(const SolveArgs a);
+template __global__ void fct_solve_kernel<128, false, 1, false>(const SolveArgs a);

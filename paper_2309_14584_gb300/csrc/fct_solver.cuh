@@ -1195,10 +1195,10 @@ __device__ bool pcg_normal_w(const DevPlan& P, Team& tm, const BlockTabs& T, dou
 // nonempty bins, then the FP64 solve, or FP64 normal-residual sweeps around
 // FP32 inner solves (mixed).
 // ---------------------------------------------------------------------------
-// Inlined at each of the kernel's three call sites (alone, batch, serving): as a
-// function its tables and team would live in local memory, whose lines every
-// barrier's acquire drops (sparse D = 100, N = 50000: 62.0 ms against 56.9).
-template <int BT, bool SV, int DEEP>
+// Inlined into the kernel: as a function its tables and team would live in local
+// memory, whose lines every barrier's acquire drops (sparse D = 100, N = 50000:
+// 62.0 ms against 56.9).
+template <int BT, bool SV, int DEEP, bool CELLS>
 __device__ __forceinline__ bool solve_job(const SolveJob& J, Team& tm, double* red, unsigned char* dsm, int smem_bytes) {
   // The plan's header in shared memory: every barrier's gpu-scope acquire drops
   // L1, so the first use after a barrier of a field held in global memory would
@@ -1221,7 +1221,7 @@ __device__ __forceinline__ bool solve_job(const SolveJob& J, Team& tm, double* r
   }
   // the inner solve by grid groups takes the whole of the block's shared memory
   // once b is known, so nothing but the DCT matrices is staged for it
-  const bool cells = !SV && J.precision == FCT_MIXED && P.tk_groups > 0 && P.s_init == nullptr;
+  const bool cells = CELLS && J.precision == FCT_MIXED && P.tk_groups > 0 && P.s_init == nullptr;
   if (cells && smem_bytes < P.tk_smem) {  // the host sizes launches to hold it
     if (threadIdx.x == 0) atomicExch(tm.err, static_cast<int>(FCT_ERR_INVALID_ARG));
     return false;
@@ -1329,7 +1329,7 @@ __device__ __forceinline__ bool solve_job(const SolveJob& J, Team& tm, double* r
         if (!pcg_normal_w<BT>(P, tm, T, g64 * ci * ci, J.inner_tol, J.max_iter, 64, &it_in, &g_in, &st_in))
           return false;
       } else if (cells) {
-        if constexpr (!SV) {
+        if constexpr (CELLS) {
           if (!cg_cells<BT>(P, tm, dsm, g64 * ci * ci, J.inner_tol, J.max_iter, 64, &it_in, &g_in, &st_in))
             return false;
         }
@@ -1418,10 +1418,11 @@ __device__ __forceinline__ bool solve_job(const SolveJob& J, Team& tm, double* r
   return true;
 }
 
-template <int BT, bool SV, int DEEP>
+template <int BT, bool SV, int DEEP, bool CELLS>
 __global__ void __launch_bounds__(BT, 512 / BT) fct_solve_kernel(const SolveArgs a) {
   __shared__ double red[BT / 32 + 2];
   __shared__ int s_job;
+  __shared__ SolveJob s_jobdesc;
   extern __shared__ __align__(16) unsigned char dsm[];
   const int team = blockIdx.x / a.team_blocks;
   Team tm;
@@ -1431,10 +1432,18 @@ __global__ void __launch_bounds__(BT, 512 / BT) fct_solve_kernel(const SolveArgs
   tm.bar = &a.ls->bars[team];
   tm.err = &a.ls->err;
   tm.timeout_ns = a.timeout_ns;
-  if (a.ring != nullptr) {
-    // Serving: claim published jobs until idle for idle_ns or asked to stop.
-    __shared__ SolveJob s_jobdesc;
-    for (;;) {
+  if constexpr (SV || DEEP > 0) {  // variants for one transform on the whole grid
+    // (a call of its own, its arguments in constant memory: D = 10 degree 8, mixed,
+    // staged: 7.82 ms through the loop below, 7.55 so)
+    if (solve_job<BT, SV, DEEP, CELLS>(a.single, tm, red, dsm, a.smem_bytes)) team_exit(tm);
+    return;
+  }
+  // Every team takes one job after another: the launch's only one, the next of a
+  // batch's queue, or (serving) the next published one until idle for idle_ns or
+  // asked to stop.  One call of solve_job for the three: it is inlined, and a copy
+  // for each would cost registers.
+  for (;;) {
+    if (a.ring != nullptr) {
       if (tm.rank == 0 && threadIdx.x == 0) {
         long long got = -1;
         const unsigned long long t0 = globaltimer_ns();
@@ -1466,65 +1475,60 @@ __global__ void __launch_bounds__(BT, 512 / BT) fct_solve_kernel(const SolveArgs
         a.ls->team_job[team] = static_cast<int>(got);
       }
       if (!team_sync(tm)) return;
-      if (threadIdx.x == 0) {
+    } else if (a.jobs != nullptr) {
+      if (tm.rank == 0 && threadIdx.x == 0) {
+        const unsigned int j = atomicAdd(&a.ls->queue_head, 1u);
+        a.ls->team_job[team] = j < static_cast<unsigned int>(a.njobs) ? static_cast<int>(j) : -1;
+      }
+      if (!team_sync(tm)) return;
+    }
+    if (threadIdx.x == 0) {
+      if (a.ring != nullptr || a.jobs != nullptr) {
         const int j = ldcg(&a.ls->team_job[team]);
         s_job = j;
-        if (j >= 0) s_jobdesc = a.ring->slots[j % kRingSize].job;
+        if (j >= 0) s_jobdesc = a.ring != nullptr ? a.ring->slots[j % kRingSize].job : a.jobs[j];
+      } else {
+        s_job = 0;
+        s_jobdesc = a.single;
       }
-      __syncthreads();
-      const int j = s_job;
-      const SolveJob J = s_jobdesc;
-      __syncthreads();
-      if (j < 0) break;
-      if (!solve_job<BT, SV, DEEP>(J, tm, red, dsm, a.smem_bytes)) {
-        // Abandoned (a bounded wait expired in this team or another one): the
-        // job is reported finished with the launch's error code, the error is
-        // published in the ring for the host, the job no longer counts as
-        // busy, and the launch winds down (the host does not relaunch it).
-        if (tm.rank == 0 && threadIdx.x == 0) {
-          const int err = ld_volatile_i32(&a.ls->err);
-          fct_report rep;
-          rep.status = err != 0 ? err : static_cast<int>(FCT_ERR_TIMEOUT);
-          rep.iterations = 0;
-          rep.refinements = 0;
-          rep.reserved = 0;
-          rep.rel_normal_residual = 0.0;
-          rep.gamma0 = 0.0;
-          *J.report = rep;
-          st_release_sys_i32(&a.ring->err, rep.status);
-          __threadfence_system();
-          st_release_sys_i32(&a.ring->slots[j % kRingSize].done, 1);
-          atomicExch(&a.ls->exiting, 1);
-          __threadfence();
-          atomicSub(&a.ls->busy, 1);
-        }
-        return;
+    }
+    __syncthreads();
+    if (s_job < 0) break;
+    if (!solve_job<BT, SV, DEEP, CELLS>(s_jobdesc, tm, red, dsm, a.smem_bytes)) {
+      // Abandoned (a bounded wait expired in this team or another one).  Serving:
+      // the job is reported finished with the launch's error code, the error is
+      // published in the ring for the host, the job no longer counts as
+      // busy, and the launch winds down (the host does not relaunch it).
+      if (a.ring != nullptr && tm.rank == 0 && threadIdx.x == 0) {
+        const int err = ld_volatile_i32(&a.ls->err);
+        fct_report rep;
+        rep.status = err != 0 ? err : static_cast<int>(FCT_ERR_TIMEOUT);
+        rep.iterations = 0;
+        rep.refinements = 0;
+        rep.reserved = 0;
+        rep.rel_normal_residual = 0.0;
+        rep.gamma0 = 0.0;
+        *s_jobdesc.report = rep;
+        st_release_sys_i32(&a.ring->err, rep.status);
+        __threadfence_system();
+        st_release_sys_i32(&a.ring->slots[s_job % kRingSize].done, 1);
+        atomicExch(&a.ls->exiting, 1);
+        __threadfence();
+        atomicSub(&a.ls->busy, 1);
       }
+      return;
+    }
+    if (a.ring != nullptr) {
       if (tm.rank == 0 && threadIdx.x == 0) {
         __threadfence_system();
-        st_release_sys_i32(&a.ring->slots[j % kRingSize].done, 1);
+        st_release_sys_i32(&a.ring->slots[s_job % kRingSize].done, 1);
         atomicExch(&a.ls->last_ns, globaltimer_ns());
         __threadfence();
         atomicSub(&a.ls->busy, 1);
       }
+    } else if (a.jobs == nullptr) {
+      break;
     }
-    team_exit(tm);
-    return;
-  }
-  if (a.jobs == nullptr) {
-    if (team == 0 && solve_job<BT, SV, DEEP>(a.single, tm, red, dsm, a.smem_bytes)) team_exit(tm);
-    return;
-  }
-  for (;;) {
-    if (tm.rank == 0 && threadIdx.x == 0) a.ls->team_job[team] = static_cast<int>(atomicAdd(&a.ls->queue_head, 1u));
-    if (!team_sync(tm)) return;
-    if (threadIdx.x == 0) s_job = ldcg(&a.ls->team_job[team]);
-    __syncthreads();
-    const int j = s_job;
-    __syncthreads();
-    if (j >= a.njobs) break;
-    if (!solve_job<BT, SV, DEEP>(a.jobs[j], tm, red, dsm, a.smem_bytes)) return;
   }
   team_exit(tm);
 }
-
