@@ -239,7 +239,7 @@ __global__ void eval_expansion_kernel(const uint16_t* __restrict__ support, cons
 }
 
 // Evaluation by shared prefixes (fct_evaluate's kernel; the one above, term by
-// term, serves supports whose stack or tables do not fit).  The nonzero components (axis, degree) of the
+// term, serves supports whose stacks or tables leave too little room, see there).  The nonzero components (axis, degree) of the
 // indices, in support order, form a trie whose node values are
 //   v(node) = T_degree(x_axis) (c_node + sum of its children's v),
 // so every node takes one multiply-add, whatever the depth: about one per term on
@@ -1223,20 +1223,25 @@ fct_status fct_evaluate(fct_plan P, const double* coeffs, int64_t npoints, const
   FCT_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
   {
     // points per block: 32 (one per lane, every word of the program uniform in a
-    // warp), fewer where their tables would leave less than two blocks per SM, or
-    // where the points would not fill the GPU and more workers have chunks to take.  Supports whose stack does not fit (very
-    // many nonzero components) are evaluated term by term below.
+    // warp), fewer where their tables and the threads' stacks would leave less than
+    // two blocks per SM, or where the points would not fill the GPU and more workers
+    // have chunks to take.  Supports that leave room for fewer than four points (many
+    // nonzero components, or long axes beside them) are evaluated term by term below:
+    // a block has at most 64 chunks to give to its 256 threads, so at one or two
+    // points most threads idle (128 axes, 3000 terms, 3000 points: 60 nonzero
+    // components 16.9 ms against 6.8 term by term, 45 components, four points per
+    // block, 1.6 against 6.8).
     const int tk = P->dmax + 1;
     auto need = [&](int pp) {
       return sizeof(double) * ((static_cast<size_t>(P->D) * tk + P->echunks) * pp +
                                static_cast<size_t>(P->edepth) * kEvalThreads);
     };
     int pp = 32;
-    while (pp > 1 && (need(pp) > static_cast<size_t>(optin) / 2 ||
-                      ((npoints + pp - 1) / pp < 304 && kEvalThreads / pp < P->echunks)))
-      pp >>= 1;
+    while (pp > 1 && need(pp) > static_cast<size_t>(optin) / 2) pp >>= 1;
+    const bool fits = pp >= 4;
+    while (pp > 1 && (npoints + pp - 1) / pp < 304 && kEvalThreads / pp < P->echunks) pp >>= 1;
     const int64_t nb = (npoints + pp - 1) / pp;
-    if (P->echunks > 0 && need(pp) <= static_cast<size_t>(optin) && nb <= 0x7fffffff) {
+    if (P->echunks > 0 && fits && nb <= 0x7fffffff) {
       FCT_CUDA(cudaFuncSetAttribute(eval_trie_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
       eval_trie_kernel<<<static_cast<unsigned>(nb), kEvalThreads, need(pp), static_cast<cudaStream_t>(stream)>>>(
           P->d_eprog, P->d_eword, P->echunks, P->N, P->D, tk, P->edepth, pp, coeffs, points, npoints, values);
