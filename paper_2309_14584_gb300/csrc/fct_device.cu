@@ -17,6 +17,7 @@
 // the elementwise updates.  All reductions are two-stage with a fixed order
 // (per-chunk block sums, then one sum over chunk partials), so a transform's
 // result does not depend on the team size or on the rest of the batch.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -251,12 +252,15 @@ __global__ void eval_expansion_kernel(const uint16_t* __restrict__ support, cons
 // cut into `chunks` programs of their own, so a block of eval_trie_threads threads
 // can give `ppb` points to each of threads / ppb workers, and the chunk sums are
 // added in chunk order: a value does not depend on how many points are asked for.
+// SPLIT (few points): a cluster of blocks shares the chunks of its points and
+// leaves the sums in its first block's shared memory.
 // Measured (term by term before): D = 6 degree 10 at 131072 points 14.2 -> 3.9 ms,
 // 1.07e9 multiply-adds at half the measured FP64 rate (the other half: the chunks'
 // restarts, the last wave, and chains of dependent multiply-adds at 40 warps per
 // SM); D = 3 degree 5 at 10955 points 18.3 -> 13.0 us (latency).
 constexpr int kEvalThreads = 256;
 
+template <bool SPLIT>
 __global__ void __launch_bounds__(kEvalThreads) eval_trie_kernel(
     const uint32_t* __restrict__ prog, const int32_t* __restrict__ chunk_word, int chunks, int64_t N, int D, int tk,
     int depth, int ppb, const double* __restrict__ coeffs, const double* __restrict__ points, int64_t P,
@@ -266,7 +270,13 @@ __global__ void __launch_bounds__(kEvalThreads) eval_trie_kernel(
   double* part = tab + static_cast<size_t>(D) * tk * ppb;             // [chunks][ppb]
   double* stk = part + static_cast<size_t>(chunks) * ppb;             // [depth][threads]
   const int tid = threadIdx.x;
-  const int64_t p0 = static_cast<int64_t>(blockIdx.x) * ppb;
+  int split = 1, rank = 0;
+  if constexpr (SPLIT) {
+    split = static_cast<int>(cooperative_groups::this_cluster().num_blocks());
+    rank = static_cast<int>(cooperative_groups::this_cluster().block_rank());
+    part = cooperative_groups::this_cluster().map_shared_rank(part, 0);
+  }
+  const int64_t p0 = static_cast<int64_t>(SPLIT ? blockIdx.x / split : blockIdx.x) * ppb;
   for (int e = tid; e < D * ppb; e += kEvalThreads) {
     const int i = e / ppb, j = e - i * ppb;
     const double x = p0 + j < P ? points[(p0 + j) * D + i] : 0.0;
@@ -281,8 +291,9 @@ __global__ void __launch_bounds__(kEvalThreads) eval_trie_kernel(
       t1 = t2;
     }
   }
-  __syncthreads();
-  const int j = tid % ppb, worker = tid / ppb, workers = kEvalThreads / ppb;
+  if constexpr (SPLIT) cooperative_groups::this_cluster().sync();  // the first block is there to be written to
+  else __syncthreads();
+  const int j = tid % ppb, worker = tid / ppb * split + rank, workers = kEvalThreads / ppb * split;
   const double* tj = tab + j;
   for (int c = worker; c < chunks; c += workers) {
     const uint32_t* w = prog + __ldg(chunk_word + c);
@@ -312,7 +323,12 @@ __global__ void __launch_bounds__(kEvalThreads) eval_trie_kernel(
     }
     part[c * ppb + j] = cur;
   }
-  __syncthreads();
+  if constexpr (SPLIT) {
+    cooperative_groups::this_cluster().sync();
+    if (rank > 0) return;
+  } else {
+    __syncthreads();
+  }
   if (tid < ppb && p0 + tid < P) {
     double v = part[tid];
     for (int c = 1; c < chunks; ++c) v += part[c * ppb + tid];
@@ -1224,28 +1240,62 @@ fct_status fct_evaluate(fct_plan P, const double* coeffs, int64_t npoints, const
   {
     // points per block: 32 (one per lane, every word of the program uniform in a
     // warp), fewer where their tables and the threads' stacks would leave less than
-    // two blocks per SM, or where the points would not fill the GPU and more workers
-    // have chunks to take.  Supports that leave room for fewer than four points (many
+    // two blocks per SM.  Supports that leave room for fewer than four points (many
     // nonzero components, or long axes beside them) are evaluated term by term below:
     // a block has at most 64 chunks to give to its 256 threads, so at one or two
     // points most threads idle (128 axes, 3000 terms, 3000 points: 60 nonzero
     // components 16.9 ms against 6.8 term by term, 45 components, four points per
     // block, 1.6 against 6.8).
+    // Where the points leave SMs idle, clusters of up to eight blocks share the
+    // chunks of their points, as long as all blocks stay resident together: D = 6
+    // degree 10, 1000 points 100.7 -> 47.2 us, 8000 points 437 -> 295 us; D = 2
+    // degree 300, 1000 points 556 -> 386 us (term by term 497); before, the blocks took
+    // fewer points, and their warps walked different programs side by side.  That is
+    // still done where the tables leave room for fewer than 32 points and the
+    // clusters would not take all chunks at once (100 axes, 3 components of degree up
+    // to 9, 20000 terms, 2000 points: 561 us so, 827 by clusters), and where the tables
+    // take longer than a chunk (D = 1 degree 700, 1000 points: 43.7 us so, 50.2).
     const int tk = P->dmax + 1;
     auto need = [&](int pp) {
       return sizeof(double) * ((static_cast<size_t>(P->D) * tk + P->echunks) * pp +
                                static_cast<size_t>(P->edepth) * kEvalThreads);
     };
-    int pp = 32;
+    int pp = 32, split = 1;
     while (pp > 1 && need(pp) > static_cast<size_t>(optin) / 2) pp >>= 1;
     const bool fits = pp >= 4;
-    while (pp > 1 && (npoints + pp - 1) / pp < 304 && kEvalThreads / pp < P->echunks) pp >>= 1;
-    const int64_t nb = (npoints + pp - 1) / pp;
-    if (P->echunks > 0 && fits && nb <= 0x7fffffff) {
-      FCT_CUDA(cudaFuncSetAttribute(eval_trie_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
-      eval_trie_kernel<<<static_cast<unsigned>(nb), kEvalThreads, need(pp), static_cast<cudaStream_t>(stream)>>>(
-          P->d_eprog, P->d_eword, P->echunks, P->N, P->D, tk, P->edepth, pp, coeffs, points, npoints, values);
-      FCT_CUDA(cudaGetLastError());
+    const int sms = P->max_coresident / P->blocks_per_sm;
+    auto blocks = [&] { return (npoints + pp - 1) / pp; };
+    if (blocks() < 2 * sms) {
+      const int64_t resident =  // an SM has 1 KB more than a block may ask for, which every block takes
+          sms * static_cast<int64_t>(std::min<size_t>(8, (static_cast<size_t>(optin) + 1024) / (need(pp) + 1024)));
+      const bool long_tables = tk * static_cast<int64_t>(P->echunks) > 2 * P->N;
+      auto chunks_left = [&] { return kEvalThreads / pp * split < P->echunks; };
+      while (!long_tables && split < 8 && chunks_left() && split * blocks() < 2 * sms &&
+             2 * split * blocks() <= resident)
+        split <<= 1;
+      if ((pp < 32 || long_tables) && chunks_left()) {
+        split = 1;
+        while (pp > 1 && chunks_left() && blocks() < 2 * sms) pp >>= 1;
+      }
+    }
+    if (P->echunks > 0 && fits && blocks() <= 0x7fffffff) {
+      const auto kernel = split > 1 ? eval_trie_kernel<true> : eval_trie_kernel<false>;
+      FCT_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
+      cudaLaunchConfig_t cfg{};
+      cfg.gridDim = dim3(static_cast<unsigned>(blocks() * split));
+      cfg.blockDim = dim3(kEvalThreads);
+      cfg.dynamicSmemBytes = need(pp);
+      cfg.stream = static_cast<cudaStream_t>(stream);
+      cudaLaunchAttribute attr[1];
+      attr[0].id = cudaLaunchAttributeClusterDimension;
+      attr[0].val.clusterDim.x = static_cast<unsigned>(split);
+      attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+      cfg.attrs = attr;
+      cfg.numAttrs = split > 1 ? 1 : 0;
+      const uint32_t* prog = P->d_eprog;
+      const int32_t* word = P->d_eword;
+      FCT_CUDA(cudaLaunchKernelEx(&cfg, kernel, prog, word, P->echunks, P->N, P->D, tk, P->edepth, pp, coeffs, points,
+                                  npoints, values));
       return FCT_OK;
     }
   }
