@@ -23,7 +23,7 @@ LIB = os.path.join(PKG, "libfct_gb300.so")
 SOURCES = ["fct_solve_k256.cu", "fct_solve_k128.cu", "fct_solve_k512.cu", "fct_solve_k256d.cu", "fct_solve_k128d.cu",
            "fct_solve_k512d.cu", "fct_solve_k256c.cu", "fct_solve_k128c.cu", "fct_solve_k512c.cu", "fct_device.cu",
            "fct_plan_device.cu", "fct_plan_host.cpp", "fct_peaks.cu", "fct_dct_tc.cu"]
-HEADERS = ["fct_internal.h", "fct_common.cuh", "fct_solver.cuh", "fct_cells.cuh"]
+HEADERS = ["fct_internal.h", "fct_df.cuh", "fct_common.cuh", "fct_solver.cuh", "fct_cells.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

@@ -411,10 +411,10 @@ __device__ bool cg_cells(const DevPlan& P, Team& tm, unsigned char* dsm, double 
   const double rs = ldexp(1.0, -(e0 / 2));  // exact scaling near 1/sqrt(gamma0)
   const float rsf = static_cast<float>(rs);
   const double c0 = gamma0 * rs * rs;
-  const float tol2 = static_cast<float>(tol * tol * c0);
+  const float2 tol2 = df_of(tol * tol * c0);
   // thread 0's state, in scaled units
   float2 gam = df_of(c0);
-  float best = gam.x;
+  float2 best = gam;
   int best_it = 0, it = 0;
   bool first = true;
   auto flush = [&](float2* part, int u0, int nk) {
@@ -441,11 +441,11 @@ __device__ bool cg_cells(const DevPlan& P, Team& tm, unsigned char* dsm, double 
             } else {
               bt = df_div(gnew, gam).x;
               gam = gnew;
-              if (gam.x <= tol2) c = 1;
+              if (!df_less(tol2, gam)) c = 1;
               else if (it >= max_iter) c = FCT_ERR_NOCONV + 16;
               else if (stall > 0) {
-                if (gam.x < best) {
-                  best = gam.x;
+                if (df_less(gam, best)) {
+                  best = gam;
                   best_it = it;
                 } else if (it - best_it >= stall) {
                   c = 1;

@@ -699,6 +699,8 @@ __device__ __forceinline__ bool sc_finite(double v) { return isfinite(v); }
 __device__ __forceinline__ bool sc_finite(float2 v) { return isfinite(v.x); }
 __device__ __forceinline__ double sc_val(double v) { return v; }
 __device__ __forceinline__ float sc_val(float2 v) { return v.x; }
+__device__ __forceinline__ bool sc_less(double a, double b) { return a < b; }
+__device__ __forceinline__ bool sc_less(float2 a, float2 b) { return df_less(a, b); }
 __device__ __forceinline__ double sc_div(double a, double b) { return a / b; }
 __device__ __forceinline__ float sc_div(float2 a, float2 b) { return df_div(a, b).x; }
 template <typename PT> __device__ __forceinline__ PT sc_of(double v);
@@ -736,10 +738,10 @@ __device__ bool cg_normal(const DevPlan& P, Team& tm, const BlockTabs& T, const 
   frexp(gamma0, &e0);
   const double rs = ldexp(1.0, -(e0 / 2));  // power of two near 1/sqrt(gamma0): exact scaling
   const double c0 = gamma0 * rs * rs;       // gamma0 in scaled units (in [1/4, 4))
-  const V tol2 = static_cast<V>(tol * tol * c0);
+  const PT tol2 = sc_of<PT>(tol * tol * c0);
   // thread 0's state (scaled gamma)
   PT gam = sc_of<PT>(c0);
-  V best = sc_val(gam);
+  PT best = gam;
   int it = 0, best_it = 0;
   bool first = true;
   // the condition probe forms A p from p itself: its start vector may have a part
@@ -794,11 +796,11 @@ __device__ bool cg_normal(const DevPlan& P, Team& tm, const BlockTabs& T, const 
             } else {
               bt = sc_div(gnew, gam);
               gam = gnew;
-              if (sc_val(gam) <= tol2) c = 1;
+              if (!sc_less(tol2, gam)) c = 1;
               else if (it >= max_iter) c = FCT_ERR_NOCONV + 16;
               else if (stall > 0) {
-                if (sc_val(gam) < best) {
-                  best = sc_val(gam);
+                if (sc_less(gam, best)) {
+                  best = gam;
                   best_it = it;
                 } else if (it - best_it >= stall) {
                   c = 1;
@@ -972,7 +974,7 @@ __device__ bool pcg_normal_w(const DevPlan& P, Team& tm, const BlockTabs& T, dou
   frexp(gamma0, &e0);
   const double rs = ldexp(1.0, -(e0 / 2));  // exact scaling near 1/sqrt(gamma0)
   const float rsf = static_cast<float>(rs);
-  const float tol2 = static_cast<float>(tol * tol * (gamma0 * rs * rs));
+  const float2 tol2 = df_of(tol * tol * (gamma0 * rs * rs));
   // (r.r, w.r) of one element as double-float pairs, exact
   auto products = [&](float r, float w) {
     const float tr = r * rsf, tw = w * rsf;
@@ -991,7 +993,7 @@ __device__ bool pcg_normal_w(const DevPlan& P, Team& tm, const BlockTabs& T, dou
   const float* const rhs = reinterpret_cast<const float*>(P.sp32);  // s, the first half
   // thread 0's state
   float2 gam_prev = make_float2(1.0f, 0.0f), al_prev = gam_prev, gam_last = df_of(gamma0 * rs * rs);
-  float best = 3.0e38f;
+  float2 best = make_float2(3.0e38f, 0.0f);
   int best_it = 0;
 
   // y[m] = sum_j W[m][j] src[j * stride] for row m of unit u (k-th unit of this block)
@@ -1103,14 +1105,14 @@ __device__ bool pcg_normal_w(const DevPlan& P, Team& tm, const BlockTabs& T, dou
         gam_last = gam;
         if (!isfinite(gam.x) || !isfinite(del.x)) {
           c = FCT_ERR_NONFINITE + 16;
-        } else if (gam.x <= tol2) {
+        } else if (!df_less(tol2, gam)) {
           c = 1;
         } else if (it >= max_iter) {
           c = FCT_ERR_NOCONV + 16;
         } else {
           if (stall > 0) {
-            if (gam.x < best) {
-              best = gam.x;
+            if (df_less(gam, best)) {
+              best = gam;
               best_it = it;
             } else if (it - best_it >= stall) {
               c = 1;
