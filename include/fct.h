@@ -224,6 +224,17 @@ fct_status fct_plan_clone(fct_plan* out, fct_plan plan);
 /* Plan geometry (host struct). */
 fct_status fct_plan_get_info(fct_plan plan, fct_plan_info* info);
 
+/* How the mixed path's inner solve of a plan is laid out when it runs by grid
+ * groups (fct_plan_info.kernel_variant 3); all zero where it runs on A and A^T
+ * or on their product. */
+typedef struct {
+  int32_t groups;          /* tasks: groups of consecutive grids, one block each     */
+  int32_t grids_per_group; /* grids of a group (the last may hold fewer)             */
+  int32_t slices;          /* slices that the coefficients are cut into              */
+  int32_t slice_coefs;     /* coefficients of a slice (the last may hold fewer)      */
+} fct_inner_layout;
+fct_status fct_plan_get_inner_layout(fct_plan plan, fct_inner_layout* layout);
+
 /* offsets host int64[K+1]: start of each grid's samples in the samples array. */
 fct_status fct_grid_offsets(fct_plan plan, int64_t* offsets);
 

@@ -1221,6 +1221,15 @@ fct_status fct_plan_get_info(fct_plan P, fct_plan_info* info) {
   return FCT_OK;
 }
 
+fct_status fct_plan_get_inner_layout(fct_plan P, fct_inner_layout* layout) {
+  if (!P || !layout) return fail(FCT_ERR_INVALID_ARG, "NULL argument");
+  layout->groups = P->hp.tk_groups;
+  layout->grids_per_group = P->hp.tk_gg;
+  layout->slices = P->hp.tk_slices;
+  layout->slice_coefs = P->hp.tk_sl;
+  return FCT_OK;
+}
+
 fct_status fct_grid_offsets(fct_plan P, int64_t* offsets) {
   if (!P || !offsets) return fail(FCT_ERR_INVALID_ARG, "NULL argument");
   std::memcpy(offsets, P->H.offsets.data(), sizeof(int64_t) * (P->K + 1));

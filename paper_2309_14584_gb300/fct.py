@@ -102,6 +102,14 @@ class fct_plan_info(ctypes.Structure):
         return {k: getattr(self, k) for k, _ in self._fields_}
 
 
+class fct_inner_layout(ctypes.Structure):
+    _fields_ = [("groups", ctypes.c_int32), ("grids_per_group", ctypes.c_int32), ("slices", ctypes.c_int32),
+                ("slice_coefs", ctypes.c_int32)]
+
+    def as_dict(self):
+        return {n: getattr(self, n) for n, _ in self._fields_}
+
+
 class FctError(RuntimeError):
     def __init__(self, status: int, msg: str):
         super().__init__(f"{status_string(status)}: {msg}")
@@ -119,6 +127,7 @@ SIGNATURES = [
     ("fct_plan_create", ctypes.c_int, [ctypes.POINTER(_P), ctypes.c_int, ctypes.c_int64, _P, ctypes.c_int, _P, _P,
                                        ctypes.POINTER(fct_options)]),
     ("fct_plan_get_info", ctypes.c_int, [_P, ctypes.POINTER(fct_plan_info)]),
+    ("fct_plan_get_inner_layout", ctypes.c_int, [_P, ctypes.POINTER(fct_inner_layout)]),
     ("fct_grid_offsets", ctypes.c_int, [_P, _P]),
     ("fct_sample", ctypes.c_int, [_P, ctypes.c_int, _P, ctypes.c_int64, _P, _P]),
     ("fct_execute", ctypes.c_int, [_P, _P, _P, _P, ctypes.POINTER(fct_report)]),
@@ -252,6 +261,12 @@ def fct_plan_get_info(plan: int) -> dict:
     info = fct_plan_info()
     _check(lib().fct_plan_get_info(plan, ctypes.byref(info)))
     return info.as_dict()
+
+
+def fct_plan_get_inner_layout(plan: int) -> dict:
+    layout = fct_inner_layout()
+    _check(lib().fct_plan_get_inner_layout(plan, ctypes.byref(layout)))
+    return layout.as_dict()
 
 
 def fct_grid_offsets(plan: int) -> np.ndarray:
