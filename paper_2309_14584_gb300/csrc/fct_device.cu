@@ -983,10 +983,10 @@ fct_status fct_plan_create(fct_plan* out, int D, int64_t N, const uint16_t* supp
   add(&hp.part_r, sizeof(double) * hp.n_row_units);
   add(&hp.part_c, sizeof(double) * hp.n_coef_chunks);
   add(&hp.q32, sizeof(float) * H.R);
-  add(&hp.sp32, sizeof(float2) * N);
+  add(&hp.sp32, sizeof(float2) * sp32_pairs(N));
   add(&hp.dx32, sizeof(float) * N);
   add(&hp.wv, sizeof(float) * (hp.n_w_units > 0 ? 6 * N : 1));
-  add(&hp.pw64, sizeof(double2) * 2 * std::max(hp.n_w_units, 1));
+  add(&hp.pw, sizeof(float4) * 2 * std::max(hp.n_w_units, 1));
   add(&P->d_sizes, sizeof(int32_t) * K * D);
   add(&P->d_offsets, sizeof(int64_t) * (K + 1));
   add(&P->d_node_off, sizeof(int32_t) * K * D);
@@ -1802,10 +1802,10 @@ fct_status fct_plan_clone(fct_plan* out, fct_plan src) {
       {reinterpret_cast<void**>(&hp.part_r), sizeof(double) * hp.n_row_units},
       {reinterpret_cast<void**>(&hp.part_c), sizeof(double) * hp.n_coef_chunks},
       {reinterpret_cast<void**>(&hp.q32), sizeof(float) * R},
-      {reinterpret_cast<void**>(&hp.sp32), sizeof(float2) * N},
+      {reinterpret_cast<void**>(&hp.sp32), sizeof(float2) * sp32_pairs(C->N)},
       {reinterpret_cast<void**>(&hp.dx32), sizeof(float) * N},
       {reinterpret_cast<void**>(&hp.wv), sizeof(float) * (hp.n_w_units > 0 ? 6 * N : 1)},
-      {reinterpret_cast<void**>(&hp.pw64), sizeof(double2) * 2 * std::max(hp.n_w_units, 1)},
+      {reinterpret_cast<void**>(&hp.pw), sizeof(float4) * 2 * std::max(hp.n_w_units, 1)},
   };
   size_t total = 0;
   for (auto& pc : pieces) total += align256(std::max<size_t>(pc.bytes, 1));
@@ -1860,7 +1860,7 @@ __global__ void noalloc_put_plan_kernel(DevPlan* dst, const DevPlan src) {
 
 // Layout of the workspace inside the array (256-byte aligned pieces).
 struct NoallocLayout {
-  size_t devplan, report, ls, y0, y1, b, rres, q, sp, part_r, part_c, q32, sp32, dx32, wv, pw64, total;
+  size_t devplan, report, ls, y0, y1, b, rres, q, sp, part_r, part_c, q32, sp32, dx32, wv, pw, total;
 };
 
 NoallocLayout noalloc_layout(const fct_plan P) {
@@ -1885,10 +1885,10 @@ NoallocLayout noalloc_layout(const fct_plan P) {
   L.part_r = take(sizeof(double) * P->hp.n_row_units);
   L.part_c = take(sizeof(double) * P->hp.n_coef_chunks);
   L.q32 = take(sizeof(float) * R);
-  L.sp32 = take(sizeof(float2) * N);
+  L.sp32 = take(sizeof(float2) * sp32_pairs(P->N));
   L.dx32 = take(sizeof(float) * N);
   L.wv = take(sizeof(float) * (P->hp.n_w_units > 0 ? 6 * N : 1));
-  L.pw64 = take(sizeof(double2) * 2 * std::max(P->hp.n_w_units, 1));
+  L.pw = take(sizeof(float4) * 2 * std::max(P->hp.n_w_units, 1));
   L.total = off;
   return L;
 }
@@ -1936,7 +1936,7 @@ extern "C" fct_status fct_execute_noalloc(fct_plan P, const double* samples, dou
   hp.sp32 = reinterpret_cast<float2*>(b + L.sp32);
   hp.dx32 = reinterpret_cast<float*>(b + L.dx32);
   hp.wv = reinterpret_cast<float*>(b + L.wv);
-  hp.pw64 = reinterpret_cast<double2*>(b + L.pw64);
+  hp.pw = reinterpret_cast<float4*>(b + L.pw);
   DevPlan* dplan = reinterpret_cast<DevPlan*>(b + L.devplan);
   fct_report* drep = reinterpret_cast<fct_report*>(b + L.report);
   LaunchState* ls = reinterpret_cast<LaunchState*>(b + L.ls);

@@ -198,7 +198,7 @@ struct DevPlan {
   double* part_c;            // [n_coef_chunks]  (|s|^2 and the refinement sweeps)
   // FP32 workspace of the mixed path
   float* q32;                // [R]
-  float2* sp32;              // [N] {s, p} of the inner FP32 solve (by grid groups and on W: s, then p)
+  float2* sp32;              // [sp32_pairs(N)] {s, p} of the inner FP32 solve (by grid groups and on W: s, then p)
   float* dx32;               // [N]
   // normal matrix W = A^T A of the mixed path's inner solve (n_w_units = 0:
   // not built; the inner solve then applies A and A^T in two phases)
@@ -210,7 +210,7 @@ struct DevPlan {
   int32_t w_rows_per_unit;   // = workers / w_lanes
   int32_t pad_w;
   float* wv;                 // [6N] w (two buffers), r, p, s, z of the pipelined CG
-  double2* pw64;             // [2 * n_w_units] partials (r.r, w.r) as double-float pairs, two buffers
+  float4* pw;                // [2 * n_w_units] partials (r.r, w.r) as double-float pairs, two buffers
   // condition estimate: when set, the FP64 solve starts from s = s_init (no
   // DCT, no b) and block 0 records (alpha_k, beta_k) of every CG iteration,
   // the Lanczos coefficients of A^T A for the start vector s_init
@@ -250,6 +250,10 @@ struct DevPlan {
   const int32_t* tk_rows;    // [K] rows of the grid
   const int32_t* tk_qoff;    // [K] start of the grid's row sums inside its group's
 };
+
+// Pairs of sp32: its halves start on 16-byte boundaries and are read in fours by the
+// inner solve by grid groups.
+inline int64_t sp32_pairs(int64_t N) { return (N + 3) / 4 * 4; }
 
 // One transform of a launch.
 struct SolveJob {

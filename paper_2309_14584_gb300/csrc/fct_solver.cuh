@@ -982,7 +982,7 @@ __device__ bool pcg_normal_w(const DevPlan& P, Team& tm, const BlockTabs& T, dou
     const float wr = __fmul_rn(tw, tr);
     return make_float4(rr.x, rr.y, wr, fmaf(tw, tr, -wr));
   };
-  float4* const pw = reinterpret_cast<float4*>(P.pw64);
+  float4* const pw = P.pw;
   float* const wb0 = P.wv;
   float* const wb1 = P.wv + N;
   float* const vr = P.wv + 2 * static_cast<size_t>(N);
