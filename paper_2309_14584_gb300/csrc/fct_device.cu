@@ -1522,18 +1522,25 @@ static fct_status batch_setup(int B, const fct_plan* plans, const double* const*
   }
   int G = team_blocks;
   if (G <= 0) {
-    // Blocks per team from a model of the launch: a CG iteration of a transform
-    // takes kIterUs of latency plus its entries over the team's threads (fitted to
-    // D = 10 degree 8 on 38..304 blocks: 18.5, 50, 101 us against 18.6, 55, 102), the
-    // iterations grow like N^(1/4) (65, 102, 180 at N = 924, 8008, 43758),
-    // the jobs go to the teams largest first, and the last team to finish counts
-    // (48 unlike transforms, mixed: 133.9 ms at the former 19 blocks, 63.9 now).
-    // A fixed share of the GPU per job leaves most of it idle once only the
-    // largest transforms of an unlike batch are left.  At most 16 teams: below a
-    // sixteenth of the GPU the model is too kind to small teams (34 small
-    // transforms: 1.75 ms on 13 blocks, 1.47 on 19).
+    // Blocks per team: the GPU shared among the jobs, sixteen at most, or the size
+    // at which a model of the launch is at least a tenth faster.  The model: a CG
+    // iteration of a transform takes kIterUs of latency plus its entries over the
+    // team's threads (fitted to D = 10 degree 8 on 38..304 blocks: 18.5, 50, 101 us
+    // against 18.6, 55, 102), the iterations grow like N^(1/4) (65, 102, 180 at N =
+    // 924, 8008, 43758), the jobs go to the teams largest first, and the last team to
+    // finish counts.  The equal share leaves most of the GPU idle once only the
+    // largest transforms of an unlike batch are left, or when the jobs are a few more
+    // than fill the teams.
+    // On 191 batches (2..128 equal transforms of D = 2..10 and 130 unlike ones, both
+    // precisions, three block sizes) this rule takes 0.75 of the share's time in the
+    // mean, 1.02 of the best measured size's; two are slower than the share by more
+    // than 2 % (by 8 % the worst).  The model alone, over every number of teams up to
+    // 16: 0.86 of the share on 101 of them, up to 1.13 (34 of D = 3 degree 6: 0.89 ms,
+    // 0.83 by shares, 0.59 now).  It is too rough to tell neighbouring sizes apart, hence
+    // the tenth and the short list of team numbers, those that were measured.
     constexpr double kIterUs = 6.5, kEntryUs = 0.717;
-    std::vector<double> work(B), iters(B);
+    constexpr int kTeamCounts[] = {1, 2, 3, 4, 6, 8, 10, 12, 13, 16, 19, 24, 32, 38};
+    std::vector<double> work(B), iters(B), busy;
     int units = 1;
     for (int q = 0; q < B; ++q) {
       const fct_plan Pq = plans[order[q]];
@@ -1542,13 +1549,7 @@ static fct_status batch_setup(int B, const fct_plan* plans, const double* const*
       iters[q] = std::sqrt(std::sqrt(static_cast<double>(Pq->N)));
       units = std::max(units, Pq->grid_blocks);
     }
-    double best = 0.0;
-    std::vector<double> busy;
-    int last = 0;
-    for (int teams = 1; teams <= std::min({B, 16, P0->max_coresident}); ++teams) {
-      const int g = std::min(units, P0->max_coresident / teams);
-      if (g == last) continue;
-      last = g;
+    auto model = [&](int g) {
       // busy: a heap whose front is the team that is free first
       busy.assign(std::min(P0->max_coresident / g, std::min(B, kMaxTeams)), 0.0);
       double t = 0.0;
@@ -1558,7 +1559,19 @@ static fct_status batch_setup(int B, const fct_plan* plans, const double* const*
         t = std::max(t, busy.back());
         std::push_heap(busy.begin(), busy.end(), std::greater<double>());
       }
-      if (G <= 0 || t < best) {
+      return t;
+    };
+    const int share = std::max(1, std::min(units, P0->max_coresident / std::min(B, 16)));
+    G = share;
+    double best = 0.9 * model(share);
+    int last = share;
+    for (const int teams : kTeamCounts) {
+      if (teams > std::min(B, P0->max_coresident)) break;
+      const int g = std::min(units, P0->max_coresident / teams);
+      if (g == last || g == share) continue;
+      last = g;
+      const double t = model(g);
+      if (t < best) {
         best = t;
         G = g;
       }

@@ -1,0 +1,56 @@
+"""The automatic team size of a batch (team_blocks = 0) against an equal share of the
+GPU for each of at most sixteen jobs: not slower on batches where a larger team only
+looks better (the times of the share were 0.88..0.95 of the automatic size's on the
+first three), much faster where the jobs are unlike."""
+import pytest
+import torch
+
+import paper_2309_14584_gb300 as F
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+# (D, degree, K) of the jobs, block threads, the share's blocks, largest ratio of the times
+CASES = {
+    "34_of_D3": ([(3, 6, 24)] * 34, 256, 19, 1.04),
+    "24_of_D3": ([(3, 6, 24)] * 24, 256, 19, 1.04),
+    "8_small_128_threads": ([(4, 9, 32)] + [(4, 6, 32), (3, 8, 24)] * 3 + [(3, 10, 24)], 128, 76, 1.06),
+    "2_of_D6_and_10_of_D3": ([(6, 10, 18)] * 2 + [(3, 6, 24)] * 10, 256, 25, 0.7),
+}
+
+
+def _time(fn):
+    fn()
+    torch.cuda.synchronize()
+    ms = []
+    for _ in range(9):
+        a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        a.record()
+        fn()
+        b.record()
+        torch.cuda.synchronize()
+        ms.append(a.elapsed_time(b))
+    return sorted(ms)[4]
+
+
+@pytest.mark.parametrize("name", CASES)
+def test_automatic_size_is_not_slower_than_an_equal_share(name):
+    jobs, bt, share, most = CASES[name]
+    base, plans, xs = {}, [], []
+    for i, (D, d, K) in enumerate(jobs):
+        if (D, d, K) in base:
+            p = base[D, d, K].clone()
+        else:
+            sup = W.total_degree_support(D, d)
+            p = base[D, d, K] = F.Plan(sup, *W.l_grid(7, len(sup), D, K, 1, d + 1), precision=F.FCT_MIXED, tol=1e-12,
+                                       inner_tol=1e-4, block_threads=bt)
+        x = torch.empty(p.M, dtype=torch.float64, device="cuda")
+        p.sample(W.FAMILY_GAUSSCOS, W.gausscos_params(1000 + i, D), x)
+        plans.append(p)
+        xs.append(x)
+    outs = [torch.empty(p.N, dtype=torch.float64, device="cuda") for p in plans]
+    hs = [p.handle for p in plans]
+    t = {g: _time(lambda: F.fct_execute_batch(hs, xs, outs, team_blocks=g, report=False)) for g in (0, share)}
+    assert t[0] <= most * t[share], t
+    for p in plans[::-1]:
+        p.close()
