@@ -725,10 +725,7 @@ fct_status fct_plan_create(fct_plan* out, int D, int64_t N, const uint16_t* supp
   P->M = H.M;
   P->sizes.assign(sizes, sizes + static_cast<size_t>(K) * D);
   int64_t nnz_support = 0;
-  for (int64_t e = 0; e < N * D; ++e) {
-    P->dmax = std::max<int>(P->dmax, support[e]);
-    nnz_support += support[e] != 0;
-  }
+  support_stats(support, N * D, &P->dmax, &nnz_support);
   // evaluation program, unless its positions leave 32 bits
   const int64_t eword_max = nnz_support + N + static_cast<int64_t>(eval_chunks(N)) * D;
   P->echunks = eword_max < (int64_t{1} << 31) ? eval_chunks(N) : 0;

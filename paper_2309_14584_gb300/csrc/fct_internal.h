@@ -462,6 +462,9 @@ struct CellPointers {
 fct_status build_cells_device(const DeviceTables& T, int64_t N, int K, const CellLayout& L, const CellPointers& out);
 void build_cells_host(const HostTables& H, const CellLayout& L, const CellPointers& out);
 
+// Largest of n components of a support, and how many are not zero.
+void support_stats(const uint16_t* support, int64_t n, int* dmax, int64_t* nonzeros);
+
 // Evaluation program of a support (eval_trie_kernel): its terms in `chunks`
 // programs of consecutive terms, chunk c starting at word[c] (word[chunks] = the
 // end, word[chunks + 1] = the most nonzero components of an index).  tk = table

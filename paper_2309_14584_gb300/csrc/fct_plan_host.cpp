@@ -544,6 +544,24 @@ void normal_matrix(const HostTables& H, std::vector<int32_t>* rowptr, std::vecto
   }
 }
 
+void support_stats(const uint16_t* support, int64_t n, int* dmax, int64_t* nonzeros) {
+  // counters of the components' own width, blocks short enough for them: the
+  // compiler takes eight components at once (N D = 437580: 189 -> 42 us on the host)
+  constexpr int64_t kBlock = 32768;
+  uint16_t most = 0;
+  *nonzeros = 0;
+  for (int64_t b = 0; b < n; b += kBlock) {
+    const int64_t end = std::min(n, b + kBlock);
+    uint16_t count = 0;
+    for (int64_t e = b; e < end; ++e) {
+      most = std::max(most, support[e]);
+      count = static_cast<uint16_t>(count + (support[e] != 0));
+    }
+    *nonzeros += count;
+  }
+  *dmax = most;
+}
+
 bool cells_pay(int64_t N, int K, int block_threads, int64_t wave) {
   return K >= wave * block_threads / 512 && N >= kCellMinN && K * N >= kCellMinEntries;
 }
