@@ -49,7 +49,8 @@ BATCH = 38                   # batched leg: transforms of the D=6 workload per l
 HETERO_BATCH = 512           # heterogeneous batch leg: transforms per launch (grid counts by Algorithm 2)
 HETERO_CHECKED = 4           # smallest transforms of the heterogeneous batch checked against the oracle
 ACCURACY_POINTS = 5000       # random points of the L-infinity error of the approximation
-SOLVER_SOURCES = ("fct_common.cuh", "fct_solver.cuh")  # hashed to match a profile to the kernel code
+# the solver kernels' code, hashed to match a profile to it
+SOLVER_SOURCES = ("fct_internal.h", "fct_df.cuh", "fct_common.cuh", "fct_solver.cuh", "fct_cells.cuh")
 HEADLINE_PROFILE = "fct_solve_kernel_D10_d8_mixed.txt"
 PATH_OPTIONS = {   # precision: 0 = FCT_FP64, 1 = FCT_MIXED (include/fct.h)
     "fp64": dict(precision=0, tol=1e-13),
@@ -326,7 +327,7 @@ class ClockSampler:
 # ---------------------------------------------------------------------------
 # roofline bookkeeping
 # ---------------------------------------------------------------------------
-def algorithmic_bytes(info, rep, precision):
+def algorithmic_bytes(info, rep, precision, layout=None):
     """Bytes the method must move per transform, with int32 tables and the
     single-point weights counted as recomputable (no stored-value bytes):
       DCT:                      8 M + 8 R    (samples in, b out)
@@ -335,11 +336,19 @@ def algorithmic_bytes(info, rep, precision):
           twice, x read and written, s written and read, p written: 8 N; q
           written and read, r read, written and gathered: 5 R)
       FP32 inner iteration:     8 K N + 4 (8 N + 5 R)
-      FP64 refinement sweep:    8 K N + 8 (8 N + 5 R)   (one A and one A^T pass)"""
+      FP64 refinement sweep:    8 K N + 8 (8 N + 5 R)   (one A and one A^T pass)
+    layout (fct_plan_get_inner_layout): a plan whose inner solve runs by G grid
+    groups streams its cell tables instead (6 bytes per entry, once to gather and
+    once to scatter) and holds the row sums in shared memory:
+      FP32 inner iteration:     12 K N + 16 G N + 24 N
+          (a group reads s and p and writes its t, 12 N; the owners read every t,
+          4 N a group, and read and write s, p and x)"""
     N, R, K, M = info["N"], info["R"], info["K"], info["M"]
     dct = 8 * M + 8 * R
     it64 = 8 * K * N + 8 * (8 * N + 5 * R)
     it32 = 8 * K * N + 4 * (8 * N + 5 * R)
+    if layout and layout["groups"]:
+        it32 = 12 * K * N + 16 * layout["groups"] * N + 24 * N
     if precision == "fp64":
         return dct + rep["iterations"] * it64
     return dct + rep["iterations"] * it32 + rep["refinements"] * it64
@@ -759,19 +768,24 @@ def approximation_error(F, plan, w, coeffs_dev) -> dict:
             "note": "max |p(x) - f(x)| of the mixed-path expansion at uniform random points"}
 
 
-def sparse_rooflines(info, rep, ms, peaks, peak_kind, gather_peak):
+def sparse_rooflines(info, rep, ms, peaks, peak_kind, gather_peak, layout=None):
     """Roofs of a sparse-support transform, whose tables (K N entries, more
     than L2 holds) are read from DRAM every iteration: the algorithmic bytes
     against the measured HBM copy rate, and the scattered loads (one per table
-    entry and alias pass) against the measured random-gather rate."""
-    bytes_ = algorithmic_bytes(info, rep, "mixed")
+    entry and alias pass) against the measured random-gather rate.  An inner
+    solve by grid groups makes its scattered accesses in shared memory, so such
+    a plan has no gather roof (None)."""
+    by_groups = bool(layout and layout["groups"])
+    bytes_ = algorithmic_bytes(info, rep, "mixed", layout)
     hbm = {"bound": "hbm", "achieved": bytes_ / (ms / 1e3) / 1e9, "peak": peaks["hbm_gbs"], "unit": "GB/s",
            "algorithmic_bytes_per_launch": bytes_,
            "peak_kind": f"{peak_kind} HBM copy bandwidth (MEASURED_PEAKS.json)",
-           "note": "table bytes counted as indices only (4 per entry and alias pass); the stored FP32 entry "
+           "note": "inner solve by grid groups: 6 table bytes per entry, read to gather and again to scatter "
+                   "(in part from L2), and the groups' vectors" if by_groups else
+                   "table bytes counted as indices only (4 per entry and alias pass); the stored FP32 entry "
                    "values double the table bytes actually read"}
     hbm["frac"] = hbm["achieved"] / hbm["peak"]
-    return hbm, gather_roofline(info, rep, ms / 1e3, gather_peak)
+    return hbm, None if by_groups else gather_roofline(info, rep, ms / 1e3, gather_peak)
 
 
 def run_next_rows(F, w, opts, flush, steps=20, large_sparse=True, gather_peak=None) -> dict:
@@ -861,7 +875,7 @@ def run_next_rows(F, w, opts, flush, steps=20, large_sparse=True, gather_peak=No
                           "refinements": rep["refinements"], "recovery_rel_err": err}
     if gather_peak:
         out["sparse_D100"]["roofline"], out["sparse_D100"]["gather_roofline"] = sparse_rooflines(
-            dict(ps.info), rep, ms, peaks, peak_kind, gather_peak)
+            dict(ps.info), rep, ms, peaks, peak_kind, gather_peak, F.fct_plan_get_inner_layout(ps.handle))
     ps.close()
     del xs, cs
     if not large_sparse:
@@ -896,7 +910,7 @@ def run_next_rows(F, w, opts, flush, steps=20, large_sparse=True, gather_peak=No
                                "refinements": rep["refinements"], "recovery_rel_err": err}
     if gather_peak:
         out["sparse_D100_N1e6"]["roofline"], out["sparse_D100_N1e6"]["gather_roofline"] = sparse_rooflines(
-            dict(pl.info), rep, ms, peaks, peak_kind, gather_peak)
+            dict(pl.info), rep, ms, peaks, peak_kind, gather_peak, F.fct_plan_get_inner_layout(pl.handle))
     pl.close()
     return out
 
