@@ -173,7 +173,7 @@ typedef struct {
   int32_t entries_per_lane; /* A p gather: entries per lane of a row unit (2, 4 or 8)   */
   int32_t kernel_variant;   /* solver kernel of fct_execute: 0 plain, 1 entry values staged
                                in shared memory, 2 deep gathers (twice the entries per
-                               lane and round), 3 plain with the mixed path's inner
+                               lane and round), 3 the same with the mixed path's inner
                                solve by grid groups                                     */
   int64_t tensor_dct_flops; /* BF16 tensor-core flops of the DCT passes per fct_execute
                                (36 digit-slice products of M 128 x N 64 x K 16 per tile

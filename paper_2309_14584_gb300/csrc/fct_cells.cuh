@@ -13,10 +13,13 @@
 //     A_l^T q_l, streamed out (tpart);
 //   phase 2, per owner chunk: t = sum over groups of tpart, then x += alpha p,
 //     s -= alpha t.
-// What bounds it now: latency and issue in the two streams (about 100 instructions
-// and 20 wavefronts of the L1 / shared-memory pipe per four steps, 8..16 warps per SM), then the
-// phases' fixed costs.  Time per CG iteration, two-matrix form -> this: sparse
-// D = 100, N = 50000, 240 grids 226 -> 70 us; N = 20000, 1000 grids 172 -> 110;
+// What bounds it now: latency in the two streams at 16 warps per SM, then the
+// phases' fixed costs.  Counters of the sparse D = 100 plans (N = 20000 on 1000
+// grids, N = 100000 on 240): DRAM at 36 and 35 % of the copy rate, issue slots 17 and
+// 18 % used, per issued instruction 10 and 9 warps at a barrier and 7 and 8 waiting for a load;
+// 81 and 98 instructions and 25 and 27 shared-memory wavefronts of the whole launch
+// per four steps of a warp.  Time per CG iteration, two-matrix form -> this: sparse
+// D = 100, N = 50000, 240 grids 226 -> 70 us; N = 20000, 1000 grids 172 -> 107;
 // D = 18 degree 5, 171 grids 56 -> 49 (171 tasks on 152 SMs).
 // Two team barriers, as in cg_normal, but every scattered access is to shared
 // memory and global traffic is coalesced: 6 bytes of table per entry (read by

@@ -419,16 +419,18 @@ fct_status cuda_fail(cudaError_t e, const char* what) {
 // CG loop's entry values in shared memory (single transforms whose tables
 // fit); kKernelDeep stages twice as many gather entries per lane and round
 // (single transforms of plans with wide rows or many grids, whose tables
-// stream from DRAM); kKernelCells is the plain one with the inner solve by grid
-// groups (plans that solve so, batches that hold one, servers).  See
-// choose_shape.
-enum { kKernelPlain = 0, kKernelStaged = 1, kKernelDeep = 2, kKernelCells = 3 };
+// stream from DRAM); kKernelCells is the deep one with the inner solve by grid
+// groups (single transforms of plans that solve so), kKernelCellsQueue the plain
+// one (batches that hold such a plan, servers).  See choose_shape.
+enum { kKernelPlain = 0, kKernelStaged = 1, kKernelDeep = 2, kKernelCells = 3, kKernelCellsQueue = 4 };
+constexpr int kKernelKinds = 5;
 
 template <int BT>
 const void* kernel_ptr(int kind) {
   if (kind == kKernelStaged) return reinterpret_cast<const void*>(&fct_solve_kernel<BT, true, 0, false>);
   if (kind == kKernelDeep) return reinterpret_cast<const void*>(&fct_solve_kernel<BT, false, 1, false>);
-  if (kind == kKernelCells) return reinterpret_cast<const void*>(&fct_solve_kernel<BT, false, 0, true>);
+  if (kind == kKernelCells) return reinterpret_cast<const void*>(&fct_solve_kernel<BT, false, 1, true>);
+  if (kind == kKernelCellsQueue) return reinterpret_cast<const void*>(&fct_solve_kernel<BT, false, 0, true>);
   return reinterpret_cast<const void*>(&fct_solve_kernel<BT, false, 0, false>);
 }
 
@@ -503,18 +505,19 @@ size_t launch_smem(const fct_plan P, int G, size_t cap) {
 // Dynamic shared memory a solver block may take without lowering the blocks
 // per SM of the plain kernel, set as the variants' limit: one value for the
 // variants without the inner solve by grid groups (the largest static shared
-// memory among them counted), at most as much for the one with it.  Plans and
+// memory among them counted), at most as much for those with it.  Plans and
 // servers of one block size compute the same values, so neither lowers the
 // other's launch limit.
 fct_status solver_smem_cap(int bt, const cudaDeviceProp& prop, int* cap_out, int* cells_cap_out, int* per_sm_out) {
   int per_sm = 0;
   FCT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, solve_kernel_for(bt), bt, 0));
   if (per_sm < 1) return fail(FCT_ERR_CUDA, "solver kernel cannot be resident");
-  size_t fixed[4];
-  for (int kind : {kKernelPlain, kKernelStaged, kKernelDeep, kKernelCells}) {
+  size_t plain = 0, cells = 0;  // largest static shared memory
+  for (int kind = 0; kind < kKernelKinds; ++kind) {
     cudaFuncAttributes fk;
     FCT_CUDA(cudaFuncGetAttributes(&fk, solve_kernel_for(bt, kind)));
-    fixed[kind] = fk.sharedSizeBytes;
+    size_t& most = kind >= kKernelCells ? cells : plain;
+    most = std::max(most, fk.sharedSizeBytes);
   }
   auto cap_for = [&](size_t sh) {
     const int reserve = 1024;  // per-block system reservation
@@ -522,12 +525,11 @@ fct_status solver_smem_cap(int bt, const cudaDeviceProp& prop, int* cap_out, int
     cap = std::min(cap, static_cast<int>(prop.sharedMemPerBlockOptin) - static_cast<int>(sh));
     return std::max(cap, 0) & ~15;
   };
-  const size_t plain = std::max({fixed[kKernelPlain], fixed[kKernelStaged], fixed[kKernelDeep]});
   *cap_out = cap_for(plain);
-  *cells_cap_out = cap_for(std::max(plain, fixed[kKernelCells]));
-  for (int kind : {kKernelPlain, kKernelStaged, kKernelDeep, kKernelCells})
+  *cells_cap_out = cap_for(std::max(plain, cells));
+  for (int kind = 0; kind < kKernelKinds; ++kind)
     FCT_CUDA(cudaFuncSetAttribute(solve_kernel_for(bt, kind), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  kind == kKernelCells ? *cells_cap_out : *cap_out));
+                                  kind >= kKernelCells ? *cells_cap_out : *cap_out));
   *per_sm_out = per_sm;
   return FCT_OK;
 }
@@ -558,9 +560,12 @@ fct_status choose_cell_layout(fct_plan P, int64_t wave, CellLayout* L) {
   FCT_CUDA(cudaGetDeviceProperties(&prop, dev));
   const fct_status s = solver_smem_cap(P->block_threads, prop, &cap, &cells_cap, &per_sm);
   if (s != FCT_OK) return s;
-  FCT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-      &cells_per_sm, solve_kernel_for(P->block_threads, kKernelCells), P->block_threads, cells_cap));
-  if (cells_per_sm >= per_sm) choose_cells(P->N, P->K, P->M, P->block_threads, wave, cells_cap, L);
+  for (int kind : {kKernelCells, kKernelCellsQueue}) {
+    FCT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&cells_per_sm, solve_kernel_for(P->block_threads, kind),
+                                                           P->block_threads, cells_cap));
+    if (cells_per_sm < per_sm) return FCT_OK;
+  }
+  choose_cells(P->N, P->K, P->M, P->block_threads, wave, cells_cap, L);
   return FCT_OK;
 }
 
@@ -1579,8 +1584,8 @@ static fct_status batch_setup(int B, const fct_plan* plans, const double* const*
   *G_out = G;
   *kind_out = kKernelPlain;
   for (int i = 0; i < B; ++i)
-    if (plans[i]->hp.tk_groups > 0) *kind_out = kKernelCells;
-  const int cap = *kind_out == kKernelCells ? P0->cells_cap : P0->smem_cap;
+    if (plans[i]->hp.tk_groups > 0) *kind_out = kKernelCellsQueue;
+  const int cap = *kind_out == kKernelCellsQueue ? P0->cells_cap : P0->smem_cap;
   size_t need = 0;
   for (int i = 0; i < B; ++i) need = std::max(need, launch_smem(plans[i], G, static_cast<size_t>(cap)));
   *smem_out = std::min(static_cast<int>(std::min<size_t>(need, cap) + 15) & ~15, cap);
@@ -2134,7 +2139,7 @@ fct_status server_ensure_running(fct_server S) {
   void* kargs[] = {&a};
   // plans of either inner solve may be submitted while the launch runs, so it is
   // the variant with both
-  FCT_CUDA(cudaLaunchCooperativeKernel(solve_kernel_for(S->block_threads, kKernelCells),
+  FCT_CUDA(cudaLaunchCooperativeKernel(solve_kernel_for(S->block_threads, kKernelCellsQueue),
                                        dim3(S->teams * S->team_blocks), dim3(S->block_threads), kargs,
                                        static_cast<size_t>(S->smem_bytes), S->stream));
   FCT_CUDA(cudaEventRecord(S->done_ev, S->stream));
