@@ -23,8 +23,9 @@
 // D = 18 degree 5, 171 grids 56 -> 49 (171 tasks on 152 SMs).
 // Two team barriers, as in cg_normal, but every scattered access is to shared
 // memory and global traffic is coalesced: 6 bytes of table per entry (read by
-// the gather and again, from L2, by the scatter) and 8 + 4 bytes of vectors per
-// coefficient and task.
+// the gather and again by the scatter; the plans above hold 120 and 144 MB of tables,
+// and both readings come from DRAM) and 8 + 4 bytes of vectors per coefficient and
+// task.
 //
 // Cell tables.  A cell is one (grid, slice of tk_sl coefficients).  Its rows are
 // cut into runs of at most kCellRun entries, sorted by length, 32 to a group:
