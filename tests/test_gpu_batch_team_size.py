@@ -26,7 +26,8 @@ def _time(fn):
     for _ in range(9):
         a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
         a.record()
-        fn()
+        for _ in range(5):
+            fn()
         b.record()
         torch.cuda.synchronize()
         ms.append(a.elapsed_time(b))
