@@ -1524,55 +1524,86 @@ static fct_status batch_setup(int B, const fct_plan* plans, const double* const*
   }
   int G = team_blocks;
   if (G <= 0) {
-    // Blocks per team: the GPU shared among the jobs, sixteen at most, or the size
-    // at which a model of the launch is at least a tenth faster.  The model: a CG
-    // iteration of a transform takes kIterUs of latency plus its entries over the
-    // team's threads (fitted to D = 10 degree 8 on 38..304 blocks: 18.5, 50, 101 us
-    // against 18.6, 55, 102), the iterations grow like N^(1/4) (65, 102, 180 at N =
-    // 924, 8008, 43758), the jobs go to the teams largest first, and the last team to
-    // finish counts.  The equal share leaves most of the GPU idle once only the
-    // largest transforms of an unlike batch are left, or when the jobs are a few more
-    // than fill the teams.
-    // On 191 batches (2..128 equal transforms of D = 2..10 and 130 unlike ones, both
-    // precisions, three block sizes) this rule takes 0.75 of the share's time in the
-    // mean, 1.02 of the best measured size's; two are slower than the share by more
-    // than 2 % (by 8 % the worst).  The model alone, over every number of teams up to
-    // 16: 0.86 of the share on 101 of them, up to 1.13 (34 of D = 3 degree 6: 0.89 ms,
-    // 0.83 by shares, 0.59 now).  It is too rough to tell neighbouring sizes apart, hence
-    // the tenth and the short list of team numbers, those that were measured.
-    constexpr double kIterUs = 6.5, kEntryUs = 0.717;
-    constexpr int kTeamCounts[] = {1, 2, 3, 4, 6, 8, 10, 12, 13, 16, 19, 24, 32, 38};
-    std::vector<double> work(B), iters(B), busy;
+    // Blocks per team, from two models of the launch: the jobs go to the teams
+    // largest first, the last team to finish counts, and a transform takes about
+    // 12.5 N^(1/4) CG iterations (8..32 N^(1/4) on 4000 transforms: no model knows
+    // better before the solve, so each choice needs a margin).
+    // The first: an iteration takes 6.5 us of latency plus its entries over the team's
+    // threads (fitted to D = 10 degree 8 on 38..304 blocks: 18.5, 50, 101 us against
+    // 18.6, 55, 102); over 1..16 teams it finds the right size for most unlike
+    // batches, where an equal share of the GPU leaves most of it idle once only the
+    // largest transforms are left.
+    // The second also counts a job's fixed cost, its samples, the barrier's growth
+    // with the team, and the rounds of row units and coefficient chunks, whose time is
+    // their load round trips: it decides between that size, the equal share (for at
+    // most 16 jobs at a time; taken on a tie), and 19, 24, 32 or 38 teams where it sees
+    // 20 % less.
+    // Measured on 137 batches of equal transforms (2..128, D = 2..18) and 220 unlike
+    // ones (3..40, D = 3..8), both precisions: in the mean 1.02 and 1.04 of the best
+    // size's time, 0.88 and 0.68 of the share's; slower than the share by more than
+    // 3 %: none and 3 (worst 1.12); of 160 unlike ones drawn after the choice 5 (worst
+    // 1.07).  The first model alone: 1.10 and 1.055 of the best,
+    // 12 and 12 slower than the share (1.47); the second alone, over all sizes: 1.01 and
+    // 1.03, but 18 unlike ones over 3 % slower than by the first (1.13).  34 of D = 3
+    // degree 6, mixed: 0.89 ms by the first model, 0.83 by shares, 0.59 now.
+    struct Job {
+      double iterations, entries, samples, fp64;  // entries per thread of a block
+      int row_units, coef_chunks;
+    };
+    std::vector<Job> model(B);
     int units = 1;
     for (int q = 0; q < B; ++q) {
       const fct_plan Pq = plans[order[q]];
-      work[q] = kEntryUs * static_cast<double>(Pq->hp.K) * static_cast<double>(Pq->N) / P0->block_threads *
-                (Pq->opt.precision == FCT_MIXED ? 1.0 : 2.0);
-      iters[q] = std::sqrt(std::sqrt(static_cast<double>(Pq->N)));
+      const double n = static_cast<double>(Pq->N);
+      model[q] = {12.5 * std::sqrt(std::sqrt(n)), Pq->hp.K * n / P0->block_threads, static_cast<double>(Pq->M),
+                  Pq->opt.precision == FCT_MIXED ? 0.0 : 1.0, Pq->hp.n_row_units, Pq->hp.n_coef_chunks};
       units = std::max(units, Pq->grid_blocks);
     }
-    auto model = [&](int g) {
+    std::vector<double> busy;
+    auto finish = [&](int g, auto job_us) {
       // busy: a heap whose front is the team that is free first
       busy.assign(std::min(P0->max_coresident / g, std::min(B, kMaxTeams)), 0.0);
       double t = 0.0;
-      for (int q = 0; q < B; ++q) {
+      for (const Job& j : model) {
         std::pop_heap(busy.begin(), busy.end(), std::greater<double>());
-        busy.back() += iters[q] * (kIterUs + work[q] / g);
+        busy.back() += job_us(j, g);
         t = std::max(t, busy.back());
         std::push_heap(busy.begin(), busy.end(), std::greater<double>());
       }
       return t;
     };
-    const int share = std::max(1, std::min(units, P0->max_coresident / std::min(B, 16)));
-    G = share;
-    double best = 0.9 * model(share);
-    int last = share;
-    for (const int teams : kTeamCounts) {
-      if (teams > std::min(B, P0->max_coresident)) break;
-      const int g = std::min(units, P0->max_coresident / teams);
-      if (g == last || g == share) continue;
+    auto first = [](const Job& j, int g) { return j.iterations * (6.5 + (1.0 + j.fp64) * 0.717 * j.entries / g); };
+    auto second = [](const Job& j, int g) {
+      const double work = 0.72 * ((j.row_units + g - 1) / g) + 1.03 * ((j.coef_chunks + g - 1) / g) + 0.717 * j.entries / g;
+      return j.iterations * (4.95 + 0.0142 * g + (1.0 + 0.47 * j.fp64) * work) + 154.0 + 0.045 * j.samples / g;
+    };
+    auto size = [&](int teams) { return std::max(1, std::min(units, P0->max_coresident / teams)); };
+    double best = 0.0;
+    int last = 0;
+    for (int teams = 1; teams <= std::min(B, 16); ++teams) {
+      const int g = size(teams);
+      if (g == last) continue;
       last = g;
-      const double t = model(g);
+      const double t = finish(g, first);
+      if (G <= 0 || t < best) {
+        best = t;
+        G = g;
+      }
+    }
+    best = finish(G, second);
+    const int share = size(std::min(B, 16));
+    if (share != G) {
+      const double t = finish(share, second);
+      if (t < 1.01 * best) {
+        best = t;
+        G = share;
+      }
+    }
+    best *= 0.8;
+    for (const int teams : {38, 32, 24, 19}) {
+      const int g = size(teams);
+      if (teams > B || g == G) continue;
+      const double t = finish(g, second);
       if (t < best) {
         best = t;
         G = g;
