@@ -722,6 +722,7 @@ __device__ bool cg_normal(const DevPlan& P, Team& tm, const BlockTabs& T, const 
   __shared__ PT wpart[kUnitGroup][NW];
   __shared__ V sh_ab[2];           // beta, alpha
   __shared__ double sh_gam;
+  __shared__ PT sh_tol2, sh_best;  // thread 0's, rarely used: not in registers
   __shared__ int sh_ctl[3];        // stop flag, status, iterations
   *status_out = FCT_OK;
   *iters_out = 0;
@@ -738,10 +739,12 @@ __device__ bool cg_normal(const DevPlan& P, Team& tm, const BlockTabs& T, const 
   frexp(gamma0, &e0);
   const double rs = ldexp(1.0, -(e0 / 2));  // power of two near 1/sqrt(gamma0): exact scaling
   const double c0 = gamma0 * rs * rs;       // gamma0 in scaled units (in [1/4, 4))
-  const PT tol2 = sc_of<PT>(tol * tol * c0);
   // thread 0's state (scaled gamma)
   PT gam = sc_of<PT>(c0);
-  PT best = gam;
+  if (threadIdx.x == 0) {
+    sh_tol2 = sc_of<PT>(tol * tol * c0);
+    sh_best = gam;
+  }
   int it = 0, best_it = 0;
   bool first = true;
   // the condition probe forms A p from p itself: its start vector may have a part
@@ -796,11 +799,11 @@ __device__ bool cg_normal(const DevPlan& P, Team& tm, const BlockTabs& T, const 
             } else {
               bt = sc_div(gnew, gam);
               gam = gnew;
-              if (!sc_less(tol2, gam)) c = 1;
+              if (!sc_less(sh_tol2, gam)) c = 1;
               else if (it >= max_iter) c = FCT_ERR_NOCONV + 16;
               else if (stall > 0) {
-                if (sc_less(gam, best)) {
-                  best = gam;
+                if (sc_less(gam, sh_best)) {
+                  sh_best = gam;
                   best_it = it;
                 } else if (it - best_it >= stall) {
                   c = 1;
